@@ -126,6 +126,7 @@ struct glbm_ctx {
     unsigned *d_status = nullptr;  // ST_WORDS status words (ST_FLAGS .. ST_HALT, glbm_internal.h)
     unsigned *h_status = nullptr;  // pinned copy of them, read after every glbm_step
     double *d_mom = nullptr;       // 7 (2D) or 9 (3D) fields of one instance
+    double *d_mw = nullptr;        // wall densities of one instance's columns (moments)
     double *d_part = nullptr;      // block partials of the conservation sums
     double *d_sums = nullptr;      // 3 sums
     double *d_diag = nullptr;      // channel diagnostics: row means and scalars
@@ -221,6 +222,14 @@ static void fill_inst(const glbm_ctx *c, const glbm_config &cfg, const Geo &g, I
         }
         ip.dew_lo[n] = slo;
         ip.dew_hi[n] = shi;
+    }
+    const AxisTableHi &tabx = tab_x(c, g);
+    for (int i = 0; i < ax_q(tabx); ++i) {
+        double vp = 1.0;
+        for (int p = 0; p < 4; ++p, vp *= ax_vel(tabx, i)) {
+            ip.kw_lo[p] += ip.ew_lo[i] * vp;
+            ip.kw_hi[p] += ip.ew_hi[i] * vp;
+        }
     }
     ip.g_theta_om = ip.g_theta / ip.omega;
     if (cfg.force == GLBM_FORCE_GUO) {
@@ -372,6 +381,7 @@ static void destroy_resources(glbm_ctx *c)
     dev_free(c->A, c->d_ip, c->stream);
     dev_free(c->A, c->d_status, c->stream);
     dev_free(c->A, c->d_mom, c->stream);
+    dev_free(c->A, c->d_mw, c->stream);
     dev_free(c->A, c->d_diag, c->stream);
     dev_free(c->A, c->d_part, c->stream);
     dev_free(c->A, c->d_sums, c->stream);
@@ -492,7 +502,7 @@ static glbm_status finish_create(glbm_ctx *c, const glbm_config *cfgs, int n, vo
     // pool layout: instances back to back, each starting on a 256-byte boundary
     c->geo.resize(n);
     long long off = 0;
-    long long max_nodes = 1;
+    long long max_nodes = 1, max_cols = 1;
     const long long align = 256 / (long long)c->elem;
     for (int i = 0; i < n; ++i) {
         Geo g = make_geo(cfgs[i]);
@@ -502,6 +512,7 @@ static glbm_status finish_create(glbm_ctx *c, const glbm_config *cfgs, int n, vo
         g.off = off;
         off += ((g.Q * g.plane + align - 1) / align) * align;
         max_nodes = std::max(max_nodes, g.nodes());
+        max_cols = std::max(max_cols, (long long)g.Lx * g.Lz);
         c->geo[i] = g;
     }
     c->pool_elems = off;
@@ -525,6 +536,7 @@ static glbm_status finish_create(glbm_ctx *c, const glbm_config *cfgs, int n, vo
     c->d_status = (unsigned *)dev_alloc(c->A, ST_WORDS * sizeof(unsigned), c->stream);
     c->d_mom = (double *)dev_alloc(c->A, (c->dims == 3 ? 9 : 7) * (size_t)max_nodes * sizeof(double),
                                    c->stream);
+    c->d_mw = (double *)dev_alloc(c->A, 2 * (size_t)max_cols * sizeof(double), c->stream);
     c->d_part = (double *)dev_alloc(c->A, 3 * (size_t)blocks * sizeof(double), c->stream);
     c->d_sums = (double *)dev_alloc(c->A, 3 * sizeof(double), c->stream);
     if (wall_rho_launch(c)) {
@@ -532,7 +544,8 @@ static glbm_status finish_create(glbm_ctx *c, const glbm_config *cfgs, int n, vo
         if (ws != GLBM_OK) return ws;
         c->wall_launch = true;
     }
-    if (!c->buf[0] || !c->buf[1] || !c->d_ip || !c->d_status || !c->d_mom || !c->d_part || !c->d_sums)
+    if (!c->buf[0] || !c->buf[1] || !c->d_ip || !c->d_status || !c->d_mom || !c->d_mw || !c->d_part ||
+        !c->d_sums)
         return fail(GLBM_E_NOMEM, "device allocation of %.1f MB failed", 2.0 * bytes_state(c) / 1e6);
     CUDA_TRY(cudaMemcpyAsync(c->d_ip, c->h_ip.data(), sizeof(InstParams) * n, cudaMemcpyHostToDevice,
                              c->stream));
@@ -1284,13 +1297,22 @@ extern "C" glbm_status glbm_sync(glbm_ctx *c)
 // ---------------------------------------------------------------------------
 // moments and conservation
 // ---------------------------------------------------------------------------
-static glbm_status compute_moments(glbm_ctx *c, int inst)
+// The fields of the mask's bits, one after another from `dst` (device memory).
+static glbm_status compute_moments(glbm_ctx *c, int inst, unsigned mask, double *dst)
 {
-    if (c->dims == 3)
-        CUDA_TRY(glbm_launch_moments3d(aux_args(c, inst), inst_ptr(c, c->cur, inst), 0, c->d_mom, c->stream));
+    const size_t nodes = (size_t)c->geo[inst].nodes();
+    MomPtrs out = {};
+    for (int b = 0; b < 9; ++b) {
+        if (!(mask & (1u << b))) continue;
+        out.p[b] = dst;
+        dst += nodes;
+    }
+    const AuxArgs a = aux_args(c, inst);
+    if (c->dims == 1)
+        CUDA_TRY(glbm_launch_moments1d(a, inst_ptr(c, c->cur, inst), out, c->stream));
     else
-        CUDA_TRY(glbm_launch_moments(aux_args(c, inst), inst_ptr(c, c->cur, inst), 0, c->d_mom, c->stream));
-    c->launches += 1;
+        CUDA_TRY(glbm_launch_moments(a, inst_ptr(c, c->cur, inst), c->d_mw, out, c->stream));
+    c->launches += c->dims > 1 && a.bc == GLBM_BC_WALLS ? 2 : 1;
     return GLBM_OK;
 }
 
@@ -1308,7 +1330,7 @@ extern "C" glbm_status glbm_channel_diagnostics(glbm_ctx *c, int inst, double *p
         c->diag_len = c->d_diag ? need : 0;
         if (!c->d_diag) return fail(GLBM_E_NOMEM, "diagnostics buffer of %zu doubles", need);
     }
-    st = compute_moments(c, inst);
+    st = compute_moments(c, inst, GLBM_M_RHO | GLBM_M_UX, c->d_mom);
     if (st != GLBM_OK) return st;
     const glbm_config &cf = c->cfg[inst];
     ChannelParams p;
@@ -1337,32 +1359,26 @@ extern "C" glbm_status glbm_moments(glbm_ctx *c, int inst, unsigned mask, double
     glbm_status st = check_inst(c, inst);
     if (st != GLBM_OK) return st;
     if (!out) return fail(GLBM_E_INVAL, "null output");
-    // field slot of each mask bit in the reducer's output
-    const int slot2d[9] = {0, 1, 2, 3, 4, 5, 6, -1, -1};
-    const int slot1d[9] = {0, 1, -1, 2, 3, -1, -1, -1, -1};
-    const int slot3d[9] = {0, 1, 2, 3, 4, 5, 6, 7, 8};
-    const int *slot = c->dims == 3 ? slot3d : (c->dims == 2 ? slot2d : slot1d);
+    // whether a field of the mask exists in this dimension
+    const unsigned has = c->dims == 3 ? GLBM_M_ALL3
+                                      : (c->dims == 2 ? GLBM_M_ALL
+                                                      : GLBM_M_RHO | GLBM_M_UX | GLBM_M_T | GLBM_M_QX);
     const size_t nodes = (size_t)c->geo[inst].nodes();
     size_t need = 0;
     if (mask >> 9) return fail(GLBM_E_INVAL, "unknown field bits in mask 0x%x", mask);
     for (int b = 0; b < 9; ++b) {
         if (!(mask & (1u << b))) continue;
-        if (slot[b] < 0) return fail(GLBM_E_INVAL, "field bit %d has no %dD meaning", b, c->dims);
+        if (!(has & (1u << b))) return fail(GLBM_E_INVAL, "field bit %d has no %dD meaning", b, c->dims);
         need += nodes;
     }
     if (need == 0) return fail(GLBM_E_INVAL, "empty field mask");
     if (out_len < need) return fail(GLBM_E_INVAL, "output holds %zu doubles, needs %zu", out_len, need);
-    st = compute_moments(c, inst);
+    st = compute_moments(c, inst, mask, out_on_device ? out : c->d_mom);
     if (st != GLBM_OK) return st;
-    size_t o = 0;
-    for (int b = 0; b < 9; ++b) {
-        if (!(mask & (1u << b))) continue;
-        CUDA_TRY(cudaMemcpyAsync(out + o, c->d_mom + (size_t)slot[b] * nodes, nodes * 8,
-                                 out_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                                 c->stream));
-        o += nodes;
+    if (!out_on_device) {
+        CUDA_TRY(cudaMemcpyAsync(out, c->d_mom, need * 8, cudaMemcpyDeviceToHost, c->stream));
+        CUDA_TRY(cudaStreamSynchronize(c->stream));
     }
-    if (!out_on_device) CUDA_TRY(cudaStreamSynchronize(c->stream));
     return GLBM_OK;
 }
 
@@ -1371,7 +1387,9 @@ extern "C" glbm_status glbm_conservation(glbm_ctx *c, int inst, double *mass, do
 {
     glbm_status st = check_inst(c, inst);
     if (st != GLBM_OK) return st;
-    st = compute_moments(c, inst);
+    st = compute_moments(c, inst,
+                         c->dims >= 2 ? GLBM_M_RHO | GLBM_M_UX | GLBM_M_UY : GLBM_M_RHO | GLBM_M_UX,
+                         c->d_mom);
     if (st != GLBM_OK) return st;
     const long long nodes = c->geo[inst].nodes();
     CUDA_TRY(glbm_launch_field_sums(c->d_mom, c->dims >= 2 ? 3 : 2, nodes, c->d_part,

@@ -1,9 +1,8 @@
 // Auxiliary kernels of libglbm: initial equilibrium, import/export of
-// populations in the FP64 logical layout, the moment reducer (moments of the
-// streamed state, Sec. 2 for rho and u; temperature, heat flux and shear
-// stress as central moments), deterministic global sums, and the 1D step
-// (Sec. 5.1 shock tube, halfway bounce-back) both per launch and resident in
-// one CTA for many steps.
+// populations in the FP64 logical layout, the 1D moment reducer (2D and 3D:
+// glbm_moments.cuh), deterministic global sums, and the 1D step (Sec. 5.1 shock
+// tube, halfway bounce-back) both per launch and resident in one CTA for many
+// steps.
 #include <algorithm>
 #include <mutex>
 
@@ -144,205 +143,52 @@ __global__ void k_get_populations(const __grid_constant__ AuxArgs a, const void 
     dst[((long long)q * a.Ly * a.Lz + y) * a.Lx + x] = v;
 }
 
-// Population of velocity (ix, iy) arriving at node (x, y) by streaming X
-// (full FP64 value), including the boundary rule. rw_lo / rw_hi are the wall
-// densities of column x.
-__device__ double pulled(const AuxArgs &a, const InstParams &ip, const void *f, long long ibase,
-                         int x, int y, int ix, int iy, double rw_lo, double rw_hi)
+// Moments of S(X) of a 1D lattice: rho, u_x, T and q_x at every node. One thread
+// per node takes the mirror pairs (+n, -n) (their sum for the even powers of xi,
+// their difference for the odd ones) with halfway bounce-back or periodic ends;
+// FP32 deviations are summed as stored and the rest weights' moments added once
+// (a reflected population has its mirror's weight). FP64 throughout.
+__global__ void k_moments1d(const __grid_constant__ AuxArgs a, const void *f, MomPtrs out)
 {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= a.Lx) return;
     const int N = a.N;
-    if (a.dims == 1) {
-        const int n = ix - N;
+    const auto pulled = [&](int n) {
         int xs = x - n;
-        int q = ix;
         if (a.bc == GLBM_BC_PERIODIC) {
-            xs = wrap_index(xs, a.Lx);
+            xs = wrap_shift(xs, a.Lx, a.Lx > N);
         } else if (xs < 0) {
             xs = -1 - xs;
-            q = 2 * N - ix;
+            n = -n;
         } else if (xs >= a.Lx) {
             xs = 2 * a.Lx - 1 - xs;
-            q = 2 * N - ix;
+            n = -n;
         }
-        double v = load_full(a, f, ibase + (long long)q * a.plane + xs, q);
-        if (a.prec != GLBM_FP64) v += a.tab.W[q];
-        return v;
+        return load_full(a, f, (long long)(N + n) * a.plane + xs, 0);
+    };
+    double R0 = pulled(0), R1 = 0.0, R2 = 0.0, R3 = 0.0, c = 0.0;
+    double w0 = a.tab.W[N], w2 = 0.0;
+    for (int n = 1; n <= N; ++n) {
+        const double vp = pulled(n), vm = pulled(-n);
+        c += 1.0;
+        const double c2 = c * c, s = vp + vm, d = c * (vp - vm), w = 2.0 * a.tab.W[N + n];
+        R0 += s;
+        R1 += d;
+        R2 = fma(c2, s, R2);
+        R3 = fma(c2, d, R3);
+        w0 += w;
+        w2 = fma(c2, w, w2);
     }
-    const int nx = ax_vel(a.tabx, ix), ny = ax_vel(a.tab, iy);
-    const int xs = wrap_index(x - nx, a.Lx);
-    int ys = y - ny;
-    if (a.bc == GLBM_BC_WALLS) {
-        if (ys < 0) return rw_lo * ip.ew_lo[ix] * a.tab.W[iy];
-        if (ys >= a.Ly) return rw_hi * ip.ew_hi[ix] * a.tab.W[iy];
-    } else {
-        ys = wrap_index(ys, a.Ly);
+    if (a.prec != GLBM_FP64) {
+        R0 += w0;
+        R2 += w2;
     }
-    const int q = iy * ax_q(a.tabx) + ix;
-    double v = load_full(a, f, ibase + (long long)q * a.plane + (long long)ys * a.pitch + xs, q);
-    if (a.prec != GLBM_FP64) v += a.tab.W[iy] * a.tabx.W[ix];
-    return v;
-}
-
-// Wall density of column x: absorbed mass / sum_{v>0} v W_v (FP64).
-__device__ double wall_density(const AuxArgs &a, const InstParams &ip, const void *f,
-                               long long ibase, int x, bool lower)
-{
-    const int N = a.N, Q1x = ax_q(a.tabx), zv = a.tab.zv;
-    double D = 0.0;
-    // velocity magnitudes |v| = m (2N+1) or 2m+1 (2N+2) in increasing order
-    for (int m = zv ? 0 : 1; m <= N; ++m) {
-        const int aa = zv ? 2 * m + 1 : m;
-        for (int k = 0; k < aa; ++k) {
-            const int iy = lower ? N - m : (zv ? N + 1 + m : N + m);
-            const int row = lower ? k : a.Ly - 1 - k;
-            for (int ix = 0; ix < Q1x; ++ix) {
-                const int xs = wrap_index(x - ax_vel(a.tabx, ix), a.Lx);
-                const int q = iy * Q1x + ix;
-                double v = load_full(a, f, ibase + (long long)q * a.plane + (long long)row * a.pitch + xs, q);
-                if (a.prec != GLBM_FP64) v += a.tab.W[iy] * a.tabx.W[ix];
-                D += v;
-            }
-        }
-    }
-    return D * ip.inv_den;
-}
-
-// out[7][Ly][Lx] (2D) or out[4][Lx] (1D): moments of S(X) at every node.
-__global__ void k_moments(const __grid_constant__ AuxArgs a, const void *f, int inst,
-                          double *__restrict__ out)
-{
-    const AxisTableHi &tx = a.dims == 2 ? a.tabx : a.tab;
-    const int Q1x = ax_q(tx);
-    const bool f64 = a.prec == GLBM_FP64;
-    // per block, from the x axis: (c, c^2, c^3) of every mirror pair's positive
-    // velocity and, for FP32 deviations, m_p = sum_ix W^x xi_x^p (the rest
-    // weights' part of a row's R_p is W^y m_p, added once per row)
-    __shared__ double cpow[GLBM_MAXQA / 2][3];
-    __shared__ double wmom[4];
-    if ((int)threadIdx.x < Q1x / 2) {
-        const double c = ax_vel(tx, Q1x - 1 - threadIdx.x), c2 = c * c;
-        cpow[threadIdx.x][0] = c;
-        cpow[threadIdx.x][1] = c2;
-        cpow[threadIdx.x][2] = c2 * c;
-    }
-    if (threadIdx.x == 32) {
-        double m0 = 0.0, m1 = 0.0, m2 = 0.0, m3 = 0.0;
-        if (!f64 && a.dims == 2) {
-            for (int ix = 0; ix < Q1x; ++ix) {
-                const double w = tx.W[ix], c = ax_vel(tx, ix);
-                m0 += w;
-                m1 = fma(c, w, m1);
-                m2 = fma(c * c, w, m2);
-                m3 = fma(c * c * c, w, m3);
-            }
-        }
-        wmom[0] = m0;
-        wmom[1] = m1;
-        wmom[2] = m2;
-        wmom[3] = m3;
-    }
-    __syncthreads();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= a.Lx) return;
-    const InstParams &ip = a.ip[inst];
-    const int Qy = a.dims == 2 ? ax_q(a.tab) : 1;
-    const int vmax = a.tab.zv ? 2 * a.N + 1 : a.N;  // fastest y velocity
-    const long long ibase = (long long)inst * a.inst_stride;
-    double rw_lo = 0.0, rw_hi = 0.0;
-    if (a.dims == 2 && a.bc == GLBM_BC_WALLS) {
-        if (y < vmax) rw_lo = wall_density(a, ip, f, ibase, x, true);
-        if (y >= a.Ly - vmax) rw_hi = wall_density(a, ip, f, ibase, x, false);
-    }
-    // one pass of raw moments, row by row: R_p = sum_ix xi_x^p v for p = 0..3,
-    // then the central moments about u from them (expanded in FP64)
-    double M0 = 0.0, jx = 0.0, jy = 0.0, Pxx = 0.0, Pyy = 0.0, Pxy = 0.0, Mx = 0.0, My = 0.0;
-    const int cmax = ax_vel(tx, Q1x - 1);  // the largest x speed
-    const bool one_wrap = a.Lx > cmax;
-    const double m0 = wmom[0], m1 = wmom[1], m2 = wmom[2], m3 = wmom[3];
-    for (int iy = 0; iy < Qy; ++iy) {
-        double R0 = 0.0, R1 = 0.0, R2 = 0.0, R3 = 0.0;
-        const int ny = a.dims == 2 ? ax_vel(a.tab, iy) : 0;
-        int ys = y - ny;
-        if (a.dims == 1 || (a.bc == GLBM_BC_WALLS && (ys < 0 || ys >= a.Ly))) {
-            // 1D (bounce-back ends) and rows emitted by a wall: value by value
-            for (int ix = 0; ix < Q1x; ++ix) {
-                const double v = pulled(a, ip, f, ibase, x, y, ix, iy, rw_lo, rw_hi);
-                const double c = ax_vel(tx, ix);
-                R0 += v;
-                R1 = fma(c, v, R1);
-                R2 = fma(c * c, v, R2);
-                R3 = fma(c * c * c, v, R3);
-            }
-        } else {
-            // a pulled row: the velocity columns in mirror pairs (+c, -c), so
-            // that the odd powers take the pair's difference and the even ones
-            // its sum; stored values (FP32: deviations) are summed and the rest
-            // weights' part is added once
-            if (a.bc != GLBM_BC_WALLS) ys = wrap_index(ys, a.Ly);
-            const long long row = ibase + (long long)(iy * Q1x) * a.plane + (long long)ys * a.pitch;
-#pragma unroll 4
-            for (int p = 0; p < Q1x / 2; ++p) {
-                const int ipos = Q1x - 1 - p;
-                const int cv = ax_vel(tx, ipos);  // > 0; column p moves at -cv
-                const long long ap = row + (long long)ipos * a.plane + wrap_shift(x - cv, a.Lx, one_wrap);
-                const long long am = row + (long long)p * a.plane + wrap_shift(x + cv, a.Lx, one_wrap);
-                const double vp = load_full(a, f, ap, 0), vm = load_full(a, f, am, 0);
-                const double sp = vp + vm, dm = vp - vm;
-                R0 += sp;
-                R1 = fma(cpow[p][0], dm, R1);
-                R2 = fma(cpow[p][1], sp, R2);
-                R3 = fma(cpow[p][2], dm, R3);
-            }
-            if (Q1x & 1) R0 += load_full(a, f, row + (long long)(Q1x / 2) * a.plane + x, 0);
-            if (!f64) {
-                const double wy = a.tab.W[iy];
-                R0 = fma(wy, m0, R0);
-                R1 = fma(wy, m1, R1);
-                R2 = fma(wy, m2, R2);
-                R3 = fma(wy, m3, R3);
-            }
-        }
-        const double cy = a.dims == 2 ? ax_vel(a.tab, iy) : 0.0;
-        M0 += R0;
-        jx += R1;
-        jy = fma(cy, R0, jy);
-        Pxx += R2;
-        Pyy = fma(cy * cy, R0, Pyy);
-        Pxy = fma(cy, R1, Pxy);
-        Mx += fma(cy * cy, R1, R3);             // sum xi_x |xi|^2 v
-        My += cy * fma(cy * cy, R0, R2);        // sum xi_y |xi|^2 v
-    }
-    const double rho = M0;
-    // u_x = (j_x + g/2) / rho with Guo's force (g_half = 0 otherwise)
-    const double ux = (jx + ip.g_half) / rho, uy = jy / rho;
-    // central second moments: P_ab - u_a j_b - j_a u_b + rho u_a u_b
-    const double cxx = Pxx - 2.0 * ux * jx + rho * ux * ux;
-    const double cyy = Pyy - 2.0 * uy * jy + rho * uy * uy;
-    const double sxy = Pxy - ux * jy - jx * uy + rho * ux * uy;
-    // sum c_a |c|^2 v, c = xi - u: M3_a - u_a tr P - 2 u.P_a + 2 u_a u.j + |u|^2 j_a - u_a |u|^2 rho
-    const double trP = Pxx + Pyy, uj = ux * jx + uy * jy, u2 = ux * ux + uy * uy;
-    const double qx = Mx - ux * trP - 2.0 * (ux * Pxx + uy * Pxy) + 2.0 * ux * uj + u2 * jx -
-                      ux * u2 * rho;
-    const double qy = My - uy * trP - 2.0 * (ux * Pxy + uy * Pyy) + 2.0 * uy * uj + u2 * jy -
-                      uy * u2 * rho;
-    const double e2 = cxx + cyy;
-    const long long plane = (long long)a.Lx * a.Ly;
-    const long long node = (long long)y * a.Lx + x;
-    if (a.dims == 2) {
-        out[0 * plane + node] = rho;
-        out[1 * plane + node] = ux;
-        out[2 * plane + node] = uy;
-        out[3 * plane + node] = e2 / (2.0 * rho);
-        out[4 * plane + node] = 0.5 * qx;
-        out[5 * plane + node] = 0.5 * qy;
-        out[6 * plane + node] = sxy;
-    } else {
-        out[0 * plane + node] = rho;
-        out[1 * plane + node] = ux;
-        out[2 * plane + node] = e2 / rho;
-        out[3 * plane + node] = 0.5 * qx;
-    }
+    const double u = R1 / R0;
+    if (out.p[0]) out.p[0][x] = R0;
+    if (out.p[1]) out.p[1][x] = u;
+    // central moments about u from the raw ones (R1 = rho u)
+    if (out.p[3]) out.p[3][x] = fma(-u, R1, R2) / R0;
+    if (out.p[4]) out.p[4][x] = 0.5 * fma(-u, 3.0 * R2 - 2.0 * (u * R1), R3);
 }
 
 // Deterministic sums of rho, rho u_x, rho u_y over n nodes: every block sums a
@@ -669,163 +515,6 @@ __global__ void k_set_equilibrium3d(const __grid_constant__ AuxArgs a, void *f, 
     }
 }
 
-// Population of velocity (ix, iy, iz) arriving at node (x, y, z) by streaming
-// X (full FP64 value), with the wall emission rho_w E^x(u_w) W^y W^z.
-__device__ double pulled3d(const AuxArgs &a, const InstParams &ip, const void *f, long long ibase,
-                           int x, int y, int z, int ix, int iy, int iz, double rw_lo, double rw_hi)
-{
-    const int N = a.N, Q1 = 2 * N + 1;
-    const int xs = wrap_index(x - (ix - N), a.Lx), zs = wrap_index(z - (iz - N), a.Lz);
-    int ys = y - (iy - N);
-    const double wyz = a.tab.W[iy] * a.tab.W[iz];
-    if (a.bc == GLBM_BC_WALLS) {
-        if (ys < 0) return rw_lo * ip.ew_lo[ix] * wyz;
-        if (ys >= a.Ly) return rw_hi * ip.ew_hi[ix] * wyz;
-    } else {
-        ys = wrap_index(ys, a.Ly);
-    }
-    const int q = (iz * Q1 + iy) * Q1 + ix;
-    double v = load_full(a, f, ibase + (long long)q * a.plane +
-                                   ((long long)zs * a.Ly + ys) * a.pitch + xs, q);
-    if (a.prec != GLBM_FP64) v += a.tab.W[ix] * wyz;
-    return v;
-}
-
-// Wall density of column (x, z): absorbed mass / sum_{n>0} n W_n.
-__device__ double wall_density3d(const AuxArgs &a, const InstParams &ip, const void *f,
-                                 long long ibase, int x, int z, bool lower)
-{
-    const int N = a.N, Q1 = 2 * N + 1;
-    double D = 0.0;
-    for (int aa = 1; aa <= N; ++aa)
-        for (int k = 0; k < aa; ++k)
-            for (int iz = 0; iz < Q1; ++iz) {
-                const int iy = lower ? N - aa : N + aa;
-                const int row = lower ? k : a.Ly - 1 - k;
-                const int zs = wrap_index(z - (iz - N), a.Lz);
-                for (int ix = 0; ix < Q1; ++ix) {
-                    const int xs = wrap_index(x - (ix - N), a.Lx);
-                    const int q = (iz * Q1 + iy) * Q1 + ix;
-                    double v = load_full(a, f, ibase + (long long)q * a.plane +
-                                                   ((long long)zs * a.Ly + row) * a.pitch + xs, q);
-                    if (a.prec != GLBM_FP64) v += a.tab.W[ix] * a.tab.W[iy] * a.tab.W[iz];
-                    D += v;
-                }
-            }
-    return D * ip.inv_den;
-}
-
-// out[9][Lz][Ly][Lx]: rho, u_x, u_y, T = sum |xi-u|^2 f / (3 rho), q_x, q_y,
-// sigma_xy, u_z, q_z of S(X).
-__global__ void k_moments3d(const __grid_constant__ AuxArgs a, const void *f, int inst,
-                            double *__restrict__ out)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int zy = blockIdx.y;
-    if (x >= a.Lx) return;
-    const int y = zy % a.Ly, z = zy / a.Ly;
-    const InstParams &ip = a.ip[inst];
-    const int N = a.N, Q1 = 2 * N + 1;
-    const long long ibase = (long long)inst * a.inst_stride;
-    double rw_lo = 0.0, rw_hi = 0.0;
-    if (a.bc == GLBM_BC_WALLS) {
-        if (y < N) rw_lo = wall_density3d(a, ip, f, ibase, x, z, true);
-        if (y >= a.Ly - N) rw_hi = wall_density3d(a, ip, f, ibase, x, z, false);
-    }
-    // one pass of raw moments, row by row (R_p = sum_ix xi_x^p v), then the
-    // central moments about u from them (expanded in FP64)
-    double rho = 0.0, jx = 0.0, jy = 0.0, jz = 0.0;
-    double Pxx = 0.0, Pyy = 0.0, Pzz = 0.0, Pxy = 0.0, Pxz = 0.0, Pyz = 0.0;
-    double Mx = 0.0, My = 0.0, Mz = 0.0;  // sum xi_a |xi|^2 v
-    const bool f64 = a.prec == GLBM_FP64;
-    const bool one_wrap = a.Lx > N;
-    // FP32 deviations: the rest weights' part of a row's R_p is W^y W^z sum_ix
-    // W^x xi_x^p, added once per row
-    double m0 = 0.0, m1 = 0.0, m2 = 0.0, m3 = 0.0;
-    if (!f64) {
-        for (int ix = 0; ix < Q1; ++ix) {
-            const double w = a.tab.W[ix], c = ix - N;
-            m0 += w;
-            m1 = fma(c, w, m1);
-            m2 = fma(c * c, w, m2);
-            m3 = fma(c * c * c, w, m3);
-        }
-    }
-    for (int iz = 0; iz < Q1; ++iz)
-        for (int iy = 0; iy < Q1; ++iy) {
-            double R0 = 0.0, R1 = 0.0, R2 = 0.0, R3 = 0.0;
-            int ys = y - (iy - N);
-            if (a.bc == GLBM_BC_WALLS && (ys < 0 || ys >= a.Ly)) {
-                // a row emitted by a wall: value by value
-                for (int ix = 0; ix < Q1; ++ix) {
-                    const double v = pulled3d(a, ip, f, ibase, x, y, z, ix, iy, iz, rw_lo, rw_hi);
-                    const double c = ix - N;
-                    R0 += v;
-                    R1 = fma(c, v, R1);
-                    R2 = fma(c * c, v, R2);
-                    R3 = fma(c * c * c, v, R3);
-                }
-            } else {
-                // a pulled row: mirror pairs (+c, -c), odd powers on the pair's
-                // difference, even ones on its sum; FP32 stores deviations, whose
-                // rest weights' part is added once per row
-                if (a.bc != GLBM_BC_WALLS) ys = wrap_index(ys, a.Ly);
-                const int zs = wrap_index(z - (iz - N), a.Lz);
-                const long long row = ibase + (long long)((iz * Q1 + iy) * Q1) * a.plane +
-                                      ((long long)zs * a.Ly + ys) * a.pitch;
-#pragma unroll 3
-                for (int n = 1; n <= N; ++n) {
-                    const double vp = load_full(a, f, row + (long long)(N + n) * a.plane +
-                                                          wrap_shift(x - n, a.Lx, one_wrap), 0);
-                    const double vm = load_full(a, f, row + (long long)(N - n) * a.plane +
-                                                          wrap_shift(x + n, a.Lx, one_wrap), 0);
-                    const double sp = vp + vm, dm = vp - vm;
-                    const double c = n, c2 = c * c;
-                    R0 += sp;
-                    R1 = fma(c, dm, R1);
-                    R2 = fma(c2, sp, R2);
-                    R3 = fma(c2 * c, dm, R3);
-                }
-                R0 += load_full(a, f, row + (long long)N * a.plane + x, 0);
-                if (!f64) {
-                    const double wyz = a.tab.W[iy] * a.tab.W[iz];
-                    R0 = fma(wyz, m0, R0);
-                    R1 = fma(wyz, m1, R1);
-                    R2 = fma(wyz, m2, R2);
-                    R3 = fma(wyz, m3, R3);
-                }
-            }
-            const double cy = iy - N, cz = iz - N, s2 = cy * cy + cz * cz;
-            rho += R0;
-            jx += R1;
-            jy = fma(cy, R0, jy);
-            jz = fma(cz, R0, jz);
-            Pxx += R2;
-            Pyy = fma(cy * cy, R0, Pyy);
-            Pzz = fma(cz * cz, R0, Pzz);
-            Pxy = fma(cy, R1, Pxy);
-            Pxz = fma(cz, R1, Pxz);
-            Pyz = fma(cy * cz, R0, Pyz);
-            Mx += fma(s2, R1, R3);
-            My += cy * fma(s2, R0, R2);
-            Mz += cz * fma(s2, R0, R2);
-        }
-    const double ux = jx / rho, uy = jy / rho, uz = jz / rho;
-    const double trP = Pxx + Pyy + Pzz, uj = ux * jx + uy * jy + uz * jz;
-    const double u2 = ux * ux + uy * uy + uz * uz;
-    const double e2 = trP - 2.0 * uj + rho * u2;
-    const double sxy = Pxy - ux * jy - jx * uy + rho * ux * uy;
-    const double uPx = ux * Pxx + uy * Pxy + uz * Pxz, uPy = ux * Pxy + uy * Pyy + uz * Pyz,
-                 uPz = ux * Pxz + uy * Pyz + uz * Pzz;
-    const double qx = Mx - ux * trP - 2.0 * uPx + 2.0 * ux * uj + u2 * jx - ux * u2 * rho;
-    const double qy = My - uy * trP - 2.0 * uPy + 2.0 * uy * uj + u2 * jy - uy * u2 * rho;
-    const double qz = Mz - uz * trP - 2.0 * uPz + 2.0 * uz * uj + u2 * jz - uz * u2 * rho;
-    const long long nodes = (long long)a.Lx * a.Ly * a.Lz;
-    const long long node = (long long)zy * a.Lx + x;
-    const double m[9] = {rho, ux, uy, e2 / (3.0 * rho), 0.5 * qx, 0.5 * qy, sxy, uz, 0.5 * qz};
-    for (int k = 0; k < 9; ++k) out[k * nodes + node] = m[k];
-}
-
 }  // namespace
 
 cudaError_t glbm_launch_set_equilibrium3d(const AuxArgs &a, void *f, int inst, const double *rho,
@@ -834,14 +523,6 @@ cudaError_t glbm_launch_set_equilibrium3d(const AuxArgs &a, void *f, int inst, c
 {
     dim3 grid((a.Lx + 127) / 128, a.Ly * a.Lz);
     k_set_equilibrium3d<<<grid, 128, 0, s>>>(a, f, inst, rho, ux, uy, uz);
-    return cudaGetLastError();
-}
-
-cudaError_t glbm_launch_moments3d(const AuxArgs &a, const void *f, int inst, double *out,
-                                  cudaStream_t s)
-{
-    dim3 grid((a.Lx + 63) / 64, a.Ly * a.Lz);
-    k_moments3d<<<grid, 64, 0, s>>>(a, f, inst, out);
     return cudaGetLastError();
 }
 
@@ -873,11 +554,10 @@ cudaError_t glbm_launch_get_populations(const AuxArgs &a, const void *f, int ins
     return cudaGetLastError();
 }
 
-cudaError_t glbm_launch_moments(const AuxArgs &a, const void *f, int inst, double *out,
-                                cudaStream_t s)
+cudaError_t glbm_launch_moments1d(const AuxArgs &a, const void *f, const MomPtrs &out,
+                                  cudaStream_t s)
 {
-    dim3 grid((a.Lx + 63) / 64, a.Ly);
-    k_moments<<<grid, 64, 0, s>>>(a, f, inst, out);
+    k_moments1d<<<(a.Lx + 31) / 32, 32, 0, s>>>(a, f, out);
     return cudaGetLastError();
 }
 

@@ -429,6 +429,17 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
     return d;
 }
 
+// (double)x by integer instructions (exact; subnormal x gives 0): a conversion
+// would take an FP64 slot, of which an SM has two per cycle.
+__device__ __forceinline__ double f2d(float x)
+{
+    const unsigned b = __float_as_uint(x), e = b & 0x7F800000u;
+    unsigned hi = ((b & 0x7FFFFFFFu) >> 3) + 0x38000000u;
+    if (e == 0x7F800000u) hi |= 0x7FF00000u;  // inf, NaN
+    hi |= b & 0x80000000u;
+    return e ? __hiloint2double((int)hi, (int)(b << 29)) : 0.0;
+}
+
 // Knuth's two-sum on both lanes (the packed form of acc2).
 __device__ __forceinline__ void acc2x2(f32x2 &s, f32x2 &c, f32x2 x)
 {

@@ -166,6 +166,7 @@ struct InstParams {
     float g_half_f;
     double dew_lo[GLBM_MAXQA];  // dE^x_i/du at u_wall_lo (2N+1 x axis; the adjoint)
     double dew_hi[GLBM_MAXQA];  // dE^x_i/du at u_wall_hi
+    double kw_lo[4], kw_hi[4];  // sum_i E^x_i(u_wall) xi_x,i^p, p = 0..3 (moments of emitted rows)
 };
 
 // Arguments of one uniform (same geometry for every instance) 2D step; TY is
@@ -293,16 +294,23 @@ cudaError_t glbm_launch_set_populations(const AuxArgs &a, void *f, int inst, con
                                         cudaStream_t s);
 cudaError_t glbm_launch_get_populations(const AuxArgs &a, const void *f, int inst, double *dst,
                                         cudaStream_t s);
-cudaError_t glbm_launch_moments(const AuxArgs &a, const void *f, int inst, double *out,
+// Destinations of the moment fields, by the bit of GLBM_M_*; null: not wanted.
+struct MomPtrs {
+    double *p[9];
+};
+// Moments of one 2D or 3D instance (f: its populations) into out[]; rw: scratch
+// for its wall densities, 2 Lx Lz doubles (unused without walls). Fields beyond
+// rho and the velocities are computed only when one of them is wanted.
+cudaError_t glbm_launch_moments(const AuxArgs &a, const void *f, double *rw, const MomPtrs &out,
                                 cudaStream_t s);
-// 3D: initial equilibrium with u_z, and the nine moment fields.
+cudaError_t glbm_launch_moments1d(const AuxArgs &a, const void *f, const MomPtrs &out,
+                                  cudaStream_t s);
+// 3D: initial equilibrium with u_z.
 cudaError_t glbm_launch_set_equilibrium3d(const AuxArgs &a, void *f, int inst, const double *rho,
                                           const double *ux, const double *uy, const double *uz,
                                           cudaStream_t s);
-cudaError_t glbm_launch_moments3d(const AuxArgs &a, const void *f, int inst, double *out,
-                                  cudaStream_t s);
 // Channel diagnostics (Sec. 5.3, 5.4) of one instance from its moment fields
-// (glbm_launch_moments / glbm_launch_moments3d output): prof[0..Ly) the row
+// (mom: rho, then u_x): prof[0..Ly) the row
 // means of u_x, prof[Ly..2Ly) of rho u_x, stats[GLBM_CH_*] the scalars.
 struct ChannelParams {
     double theta_y, tau, g;  // lattice temperature of the y axis, relaxation time, force
