@@ -25,259 +25,434 @@
 //             dE^x_i/du(u_w) W^y_i,
 // with rho_w,t from X_t: the step of time t adds its term at the wall rows,
 // k_adj_final_walls the term of F_T.
-#include "glbm_device.cuh"
+//
+// What bounds the adjoint step: the FP64 pipe (two instructions per cycle and SM;
+// mu is FP64, and a step's 79 MB at D2Q121 256 x 128 stay in L2). So the kernel
+// keeps a node's lambda and F in registers (one pull of each instead of three and
+// two), deals its velocity rows to G warps, sums the forward moments of FP32
+// states in integers (glbm_moments.cuh), evaluates each equilibrium slope once per
+// node, and forms every contraction from row sums: with d = E - W per axis,
+//   sum_i lambda E^x   = sum lambda d^x + sum lambda W^x   (per row),
+//   lambda . (f^eq - f) = rho E^y sum lambda d^x + B sum lambda W^x - sum lambda delta,
+//   B = rho E^y - W^y, delta = f - W,
+// five FP64 instructions per population for all contractions and two for mu_t, no
+// term larger than the deviations. The wall sums of mu and the wall densities of
+// X_t have a launch of their own (once per column, spread over the chip). D2Q121
+// 256 x 128, FP32 states, GB300, per step: 350 -> 103 us, the wall sums 65 -> 6 us.
+#include "glbm_moments.cuh"
 
 namespace {
 
-// E_n and dE_n/du (n = -N..N) at velocity u, FP64, from the even/odd table.
+// E_{+-n}(u) - W_n and dE_{+-n}/du of one |n| in FP64, from the even/odd table.
 template <int N>
-__device__ __forceinline__ void eq_and_slope(const AxisTable &t, double u, double (&E)[2 * N + 1],
-                                             double (&dE)[2 * N + 1])
+__device__ __forceinline__ void eq_and_slope(const AxisTable &t, int n, double u, double &dp,
+                                             double &dm, double &sp, double &sm)
 {
     const double v = u * u;
+    // Ae(v) = sum_{i=1..N} Ce[n][i] v^i and its derivative in v
+    double a = t.Ce[n][N], da = 0.0;
 #pragma unroll
-    for (int n = 0; n <= N; ++n) {
-        // Ae(v) = sum_{i=1..N} Ce[n][i] v^i and its derivative in v
-        double a = t.Ce[n][N], da = 0.0;
-#pragma unroll
-        for (int i = N - 1; i >= 1; --i) {
-            da = fma(da, v, a);
-            a = fma(a, v, t.Ce[n][i]);
-        }
-        // a now is sum_{i>=1} Ce v^(i-1); Ae = a v, Ae' = a + v da
-        const double Ae = a * v, dAe = fma(v, da, a);
-        double b = 0.0, db = 0.0;
-        if (n > 0) {
-            b = t.Co[n][N - 1];
-#pragma unroll
-            for (int i = N - 2; i >= 0; --i) {
-                db = fma(db, v, b);
-                b = fma(b, v, t.Co[n][i]);
-            }
-        }
-        // E_{+-n} = W + Ae(v) +- u Bo(v);  dE/du = 2u Ae'(v) +- (Bo + 2v Bo'(v))
-        const double odd = u * b, dodd = fma(2.0 * v, db, b);
-        E[N + n] = t.W[N + n] + Ae + odd;
-        dE[N + n] = 2.0 * u * dAe + dodd;
-        if (n > 0) {
-            E[N - n] = t.W[N - n] + Ae - odd;
-            dE[N - n] = 2.0 * u * dAe - dodd;
-        }
+    for (int i = N - 1; i >= 1; --i) {
+        da = fma(da, v, a);
+        a = fma(a, v, t.Ce[n][i]);
     }
+    // a now is sum_{i>=1} Ce v^(i-1); Ae = a v, Ae' = a + v da
+    const double Ae = a * v, sa = 2.0 * u * fma(v, da, a);
+    if (n == 0) {
+        dp = dm = Ae;
+        sp = sm = sa;
+        return;
+    }
+    double b = t.Co[n][N - 1], db = 0.0;
+#pragma unroll
+    for (int i = N - 2; i >= 0; --i) {
+        db = fma(db, v, b);
+        b = fma(b, v, t.Co[n][i]);
+    }
+    // E_{+-n} - W = Ae(v) +- u Bo(v);  dE/du = 2u Ae'(v) +- (Bo + 2v Bo'(v))
+    const double so = fma(2.0 * v, db, b);
+    dp = fma(u, b, Ae);
+    dm = fma(-u, b, Ae);
+    sp = sa + so;
+    sm = sa - so;
 }
 
-template <typename TF>
-__device__ __forceinline__ double fwd_value(const AdjArgs &a, long long idx, int iy, int ix)
-{
-    double v = (double)static_cast<const TF *>(a.X)[idx];
-    if (sizeof(TF) == 4) v += a.tab.W[iy] * a.tab.W[ix];  // FP32 stores deviations
-    return v;
-}
+// Sums over the two walls' columns before an adjoint step, a CTA of ADJ_WX columns x
+// ADJ_WS slices per wall and quantity (blockIdx.y): 0, 1 the densities rho_w of
+// the forward state X_t (lower, upper wall), 2, 3 the wall sums G(x) of mu_{t+1}.
+// The slices' partial sums are added in a fixed order.
+constexpr int ADJ_WX = 8, ADJ_WS = 32;
 
-// Wall density of column x from the forward state (FP64 sum of the absorbed mass).
 template <int N, typename TF>
-__device__ double fwd_wall_density(const AdjArgs &a, int x, bool lower)
+__global__ void __launch_bounds__(ADJ_WX *ADJ_WS) k_adj_walls(const __grid_constant__ AdjArgs a)
 {
     constexpr int Q1 = 2 * N + 1;
+    __shared__ double part[ADJ_WS][ADJ_WX];
+    wait_prior_grid();
+    const int tx = threadIdx.x % ADJ_WX, sl = threadIdx.x / ADJ_WX;
+    const int x = blockIdx.x * ADJ_WX + tx, xc = x < a.Lx ? x : a.Lx - 1;
+    const bool lower = !(blockIdx.y & 1), dens = blockIdx.y < 2;
+    const InstParams &ip = *a.ip;
     double D = 0.0;
-    for (int aa = 1; aa <= N; ++aa) {
-        for (int k = 0; k < aa; ++k) {
-            const int iy = lower ? N - aa : N + aa;
-            const int row = lower ? k : a.Ly - 1 - k;
-            for (int ix = 0; ix < Q1; ++ix) {
-                const int xs = wrap_index(x - (ix - N), a.Lx);
-                D += fwd_value<TF>(a, (long long)(iy * Q1 + ix) * a.plane + (long long)row * a.pitch + xs,
-                                   iy, ix);
-            }
+    for (int i = sl; i < N * (N + 1) / 2; i += ADJ_WS) {
+        int m = 1, k = i;  // speed |xi_y| and row
+        while (k >= m) k -= m++;
+        const int row = lower ? k : a.Ly - 1 - k;
+        if (dens) {  // absorbed by the wall
+            const int iy = lower ? N - m : N + m;
+            const TF *const p = static_cast<const TF *>(a.X) + (long long)iy * Q1 * a.plane +
+                                (long long)row * a.pitch;
+#pragma unroll
+            for (int ix = 0; ix < Q1; ++ix)
+                D += to_f64(p[(long long)ix * a.plane + wrap_shift(xc - (ix - N), a.Lx, a.Lx > N)]);
+        } else {  // emitted by the wall: velocity away from it
+            const int iy = lower ? N + m : N - m;
+            const double *const p =
+                a.mu_in + (long long)iy * Q1 * a.plane + (long long)row * a.pitch + xc;
+            double r = 0.0;
+#pragma unroll
+            for (int ix = 0; ix < Q1; ++ix)
+                r = fma(p[(long long)ix * a.plane], lower ? ip.ew_lo[ix] : ip.ew_hi[ix], r);
+            D = fma(r, a.tab.W[iy], D);
         }
     }
-    return D * a.ip->inv_den;
-}
-
-// Forward pulled population F_t,i at (x, y) (ghosts from the wall densities).
-template <int N, typename TF>
-__device__ __forceinline__ double fwd_pull(const AdjArgs &a, int x, int y, int ix, int iy,
-                                           double rw_lo, double rw_hi)
-{
-    constexpr int Q1 = 2 * N + 1;
-    const int xs = wrap_index(x - (ix - N), a.Lx);
-    int ys = y - (iy - N);
-    if (a.bc == GLBM_BC_WALLS) {
-        if (ys < 0) return rw_lo * a.ip->ew_lo[ix] * a.tab.W[iy];
-        if (ys >= a.Ly) return rw_hi * a.ip->ew_hi[ix] * a.tab.W[iy];
-    } else {
-        ys = wrap_index(ys, a.Ly);
+    part[sl][tx] = D;
+    __syncthreads();
+    for (int st = ADJ_WS / 2; st > 0; st >>= 1) {
+        if (sl < st) part[sl][tx] += part[sl + st][tx];
+        __syncthreads();
     }
-    return fwd_value<TF>(a, (long long)(iy * Q1 + ix) * a.plane + (long long)ys * a.pitch + xs, iy, ix);
+    if (sl == 0 && x < a.Lx) {
+        double v = part[0][tx] * ip.inv_den;
+        if (dens && sizeof(TF) == 4) v += 1.0;  // FP32 stores deviations
+        // G is stored over den, as the pull of an absorbed lambda takes it
+        a.walls[(long long)blockIdx.y * a.Lx + x] = v;
+    }
 }
 
-// lambda_{t+1,i} at (x, y) = (S^T mu_{t+1})_i: reverse pull from the node the
-// population streams to, or the wall term when it streams into a wall.
+// Warps a node's velocity rows are dealt to (three rows per warp: lambda and F stay
+// in registers) and CTAs per SM asked for, 15 or 16 warps where 8 left the FP64
+// pipe 61 % busy between the kernel's barriers (D2Q121 256 x 128: 128 us with 8
+// warps, 103 us with 16; two rows per warp or more warps ran no faster).
 template <int N>
-__device__ __forceinline__ double adj_pull(const AdjArgs &a, int x, int y, int ix, int iy)
-{
-    constexpr int Q1 = 2 * N + 1;
-    const int xd = wrap_index(x + (ix - N), a.Lx);
-    int yd = y + (iy - N);
-    if (a.bc == GLBM_BC_WALLS) {
-        if (yd < 0) return a.G[xd] * a.ip->inv_den;
-        if (yd >= a.Ly) return a.G[a.Lx + xd] * a.ip->inv_den;
-    } else {
-        yd = wrap_index(yd, a.Ly);
-    }
-    return a.mu_in[(long long)(iy * Q1 + ix) * a.plane + (long long)yd * a.pitch + xd];
-}
-
-// G(x) of both walls from mu_{t+1}: one thread per column.
+constexpr int ADJ_G = N == 1 ? 1 : N == 2 ? 2 : N <= 4 ? 3 : N == 5 ? 4 : N <= 7 ? 5 : 6;
 template <int N>
-__global__ void k_adj_wall(const __grid_constant__ AdjArgs a)
-{
-    constexpr int Q1 = 2 * N + 1;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= a.Lx) return;
-    double glo = 0.0, ghi = 0.0;
-    for (int ny = 1; ny <= N; ++ny) {
-        const double wy = a.tab.W[N + ny];
-        for (int k = 0; k < ny; ++k) {
-            for (int ix = 0; ix < Q1; ++ix) {
-                // emitted by the lower wall: velocity +ny into rows 0..ny-1
-                glo += a.mu_in[(long long)((N + ny) * Q1 + ix) * a.plane + (long long)k * a.pitch + x] *
-                       a.ip->ew_lo[ix] * wy;
-                // emitted by the upper wall: velocity -ny into rows Ly-ny..Ly-1
-                ghi += a.mu_in[(long long)((N - ny) * Q1 + ix) * a.plane +
-                               (long long)(a.Ly - 1 - k) * a.pitch + x] *
-                       a.ip->ew_hi[ix] * wy;
-            }
-        }
-    }
-    a.Gw[x] = glo;
-    a.Gw[a.Lx + x] = ghi;
-}
-
-constexpr int ADJ_THREADS = 64;
+constexpr int ADJ_CTAS = N == 1 ? 12 : N == 2 ? 8 : N <= 4 ? 5 : N == 5 ? 4 : N <= 7 ? 3 : 2;
 
 template <int N, typename TF>
-__global__ void __launch_bounds__(ADJ_THREADS) k_adj_step(const __grid_constant__ AdjArgs a)
+__global__ void __launch_bounds__(32 * ADJ_G<N>, ADJ_CTAS<N>)
+    k_adj_step(const __grid_constant__ AdjArgs a)
 {
-    constexpr int Q1 = 2 * N + 1;
-    __shared__ double red[GLBM_ADJ_NG][ADJ_THREADS];
-    const int x = blockIdx.x * ADJ_THREADS + threadIdx.x;
-    const int y = blockIdx.y;
+    constexpr int Q1 = 2 * N + 1, G = ADJ_G<N>, RPG = (Q1 + G - 1) / G;
+    constexpr bool DEV = sizeof(TF) == 4;
+    using ACC = std::conditional_t<DEV, MomAccI<2, N, 0, false>, MomAccD<2, N, 0, false>>;
+    __shared__ double eq[4][Q1][32];   // d^x, dE^x, d^y, dE^y
+    __shared__ double con[G][5][32];   // the groups' partial moments, then contractions
+    __shared__ double rup[3][32];      // rho - 1, u_x, u_y
+    __shared__ double tot[5][32];      // the contractions' totals
+    wait_prior_grid();
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int x = blockIdx.x * 32 + lane, y = blockIdx.y;
     const bool active = x < a.Lx;
     const int xc = active ? x : a.Lx - 1;
     const InstParams &ip = *a.ip;
-    const double om = ip.omega;
-    const double theta = N / 3.0;
+    const bool walls = a.bc == GLBM_BC_WALLS;
+    const int plane = (int)a.plane;  // Q plane < 2^31 (checked at creation)
 
+    int xs[Q1];  // source column of velocity column ix; the mirror's is its target
+#pragma unroll
+    for (int ix = 0; ix < Q1; ++ix) xs[ix] = wrap_shift(xc - (ix - N), a.Lx, a.Lx > N);
     double rw_lo = 0.0, rw_hi = 0.0;
-    if (a.bc == GLBM_BC_WALLS) {
-        if (y < N) rw_lo = fwd_wall_density<N, TF>(a, xc, true);
-        if (y >= a.Ly - N) rw_hi = fwd_wall_density<N, TF>(a, xc, false);
-    }
-    // forward moments of F_t at this node
-    double rho = 0.0, jx = 0.0, jy = 0.0;
-    for (int iy = 0; iy < Q1; ++iy)
-        for (int ix = 0; ix < Q1; ++ix) {
-            const double f = fwd_pull<N, TF>(a, xc, y, ix, iy, rw_lo, rw_hi);
-            rho += f;
-            jx += (ix - N) * f;
-            jy += (iy - N) * f;
-        }
-    const double ux = jx / rho, uy = jy / rho;
-    double Ex[Q1], dEx[Q1], Ey[Q1], dEy[Q1];
-    eq_and_slope<N>(a.tab, ux, Ex, dEx);
-    eq_and_slope<N>(a.tab, uy, Ey, dEy);
+    if (walls && y < N) rw_lo = a.walls[xc];
+    if (walls && y >= a.Ly - N) rw_hi = a.walls[a.Lx + xc];
 
+    // F_t and lambda_{t+1} of this group's rows iy = g + k G: F pulled from the node
+    // a population comes from, lambda from the node it streams to; a row out of
+    // the walls loads the edge row's F (replaced by the emission below) and takes
+    // the wall's G for lambda
+    TF f[RPG][Q1];
+    double lam[RPG][Q1];
+    const TF *const X = static_cast<const TF *>(a.X);
+#pragma unroll
+    for (int k = 0; k < RPG; ++k) {
+        const int iy = g + k * G;
+        if (iy < Q1) {
+            const int cy = iy - N;
+            int ys = y - cy, yd = y + cy;
+            const bool absorbed = walls && (yd < 0 || yd >= a.Ly);
+            const double *lp = a.walls + (yd < 0 ? 2 : 3) * (long long)a.Lx;
+            int lstep = 0;
+            if (walls) {
+                ys = min(max(ys, 0), a.Ly - 1);
+            } else {
+                ys = wrap_shift(ys, a.Ly, a.Ly > N);
+                yd = wrap_shift(yd, a.Ly, a.Ly > N);
+            }
+            if (!absorbed) {
+                lp = a.mu_in + (iy * Q1 * plane + yd * a.pitch);
+                lstep = plane;
+            }
+            const TF *const p = X + (iy * Q1 * plane + ys * a.pitch);
+#pragma unroll
+            for (int ix = 0; ix < Q1; ++ix) f[k][ix] = p[ix * plane + xs[ix]];
+#pragma unroll
+            for (int ix = 0; ix < Q1; ++ix) lam[k][ix] = lp[ix * lstep + xs[Q1 - 1 - ix]];
+        }
+    }
+
+    // forward moments (deviations of rho in FP32)
+    ACC acc;
+    acc.init();
+    double em[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < RPG; ++k) {
+        const int iy = g + k * G;
+        if (iy < Q1) {
+            const int cy = iy - N;
+            if (walls && (y - cy < 0 || y - cy >= a.Ly)) {  // emitted by a wall
+                const bool lo = y - cy < 0;
+                const double wy = a.tab.W[iy], rw = lo ? rw_lo : rw_hi;
+                const double R0 = wy * (rw * (lo ? ip.kw_lo[0] : ip.kw_hi[0]) - (DEV ? 1.0 : 0.0));
+                em[0] += R0;
+                em[1] = fma(wy * rw, lo ? ip.kw_lo[1] : ip.kw_hi[1], em[1]);
+                em[2] = fma((double)cy, R0, em[2]);
+            } else if constexpr (DEV) {
+                acc.row(f[k], cy, 0);
+            } else {
+                acc.row(f[k], (double)cy, 0.0);
+            }
+        }
+    }
+    {
+        double m[3];
+        bool ok = true;
+        if constexpr (DEV) {
+            ok = acc.in_range();
+#pragma unroll
+            for (int k = 0; k < 3; ++k) m[k] = acc.total(k);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) m[k] = acc.m[k];
+        }
+        if (!ok) {  // a deviation outside the digits' range: in FP64
+            MomAccD<2, N, 0, false> slow;
+            slow.init();
+#pragma unroll 1
+            for (int iy = g; iy < Q1; iy += G) {
+                const int ys = y - (iy - N);
+                if (walls && (ys < 0 || ys >= a.Ly)) continue;
+                const TF *const p = X + (iy * Q1 * plane +
+                                         (walls ? ys : wrap_shift(ys, a.Ly, a.Ly > N)) * a.pitch);
+                TF v[Q1];
+#pragma unroll
+                for (int ix = 0; ix < Q1; ++ix) v[ix] = p[ix * plane + xs[ix]];
+                slow.row(v, (double)(iy - N), 0.0);
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) m[k] = slow.m[k];
+        }
+        if (walls && (y < N || y >= a.Ly - N)) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) m[k] += em[k];
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) con[g][k][lane] = m[k];
+    }
+    __syncthreads();
+    if (g == 0) {
+        double m[3] = {con[0][0][lane], con[0][1][lane], con[0][2][lane]};
+#pragma unroll
+        for (int t = 1; t < G; ++t) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) m[k] += con[t][k][lane];
+        }
+        const double rho = DEV ? 1.0 + m[0] : m[0], inv = 1.0 / rho;
+        rup[0][lane] = DEV ? m[0] : m[0] - 1.0;
+        rup[1][lane] = mom_div(m[1], rho, inv);
+        rup[2][lane] = mom_div(m[2], rho, inv);
+    }
+    __syncthreads();
+    const double drho = rup[0][lane], rho = 1.0 + drho, ux = rup[1][lane], uy = rup[2][lane];
+    // the equilibrium and its slopes: group g evaluates the (|n|, axis) pairs g,
+    // g + G, ...
+#pragma unroll
+    for (int n = 0; n <= N; ++n) {
+#pragma unroll
+        for (int ax = 0; ax < 2; ++ax) {
+            if ((2 * n + ax) % G != g) continue;
+            double dp, dm, sp, sm;
+            eq_and_slope<N>(a.tab, n, ax ? uy : ux, dp, dm, sp, sm);
+            eq[2 * ax][N - n][lane] = dm;
+            eq[2 * ax + 1][N - n][lane] = sm;
+            eq[2 * ax][N + n][lane] = dp;
+            eq[2 * ax + 1][N + n][lane] = sp;
+        }
+    }
+    __syncthreads();
     // contractions of lambda_{t+1} with the equilibrium and its slopes
     double a0 = 0.0, ax = 0.0, ay = 0.0, gt = 0.0, gg = 0.0;
-    for (int iy = 0; iy < Q1; ++iy)
-        for (int ix = 0; ix < Q1; ++ix) {
-            const double lam = adj_pull<N>(a, xc, y, ix, iy);
-            const double f = fwd_pull<N, TF>(a, xc, y, ix, iy, rw_lo, rw_hi);
-            const double E = Ex[ix] * Ey[iy];
-            a0 = fma(lam, E, a0);
-            ax = fma(lam, dEx[ix] * Ey[iy], ax);
-            ay = fma(lam, Ex[ix] * dEy[iy], ay);
-            gt = fma(lam, rho * E - f, gt);
-            gg = fma(lam, a.tab.W[ix] * a.tab.W[iy] * (ix - N), gg);
-        }
-    // mu_t = (dC/dF)^T lambda at this node (the density cancels: d f^eq_i / d f_j =
-    // E_i + sum_a dE_i/du_a (xi_j,a - u_a))
-    // and the wall speeds' term of F_t: mu_t of every ghost this node pulls
-    // from a wall, times rho_w dE^x/du(u_w) W^y
-    double glo = 0.0, ghi = 0.0;
-    if (active) {
-        for (int iy = 0; iy < Q1; ++iy)
+#pragma unroll
+    for (int k = 0; k < RPG; ++k) {
+        const int iy = g + k * G;
+        if (iy < Q1) {
+            double Ld = 0.0, Lw = 0.0, Ls = 0.0, Lg = 0.0, Lf = 0.0;
+            const double wy = a.tab.W[iy];
+            const int ys = y - (iy - N);
+            const bool ghost = walls && (ys < 0 || ys >= a.Ly);
+#pragma unroll
             for (int ix = 0; ix < Q1; ++ix) {
-                const double lam = adj_pull<N>(a, xc, y, ix, iy);
-                const double m = (1.0 - om) * lam +
-                                 om * (a0 + ax * ((ix - N) - ux) + ay * ((iy - N) - uy));
-                a.mu_out[(long long)(iy * Q1 + ix) * a.plane + (long long)y * a.pitch + x] = m;
-                if (a.bc == GLBM_BC_WALLS) {
-                    const int ys = y - (iy - N);
-                    if (ys < 0) glo = fma(m * rw_lo * ip.dew_lo[ix], a.tab.W[iy], glo);
-                    if (ys >= a.Ly) ghi = fma(m * rw_hi * ip.dew_hi[ix], a.tab.W[iy], ghi);
+                const double l = lam[k][ix];
+                Ld = fma(l, eq[0][ix][lane], Ld);
+                Ls = fma(l, eq[1][ix][lane], Ls);
+                Lw = fma(l, a.tab.W[ix], Lw);
+                if (ix != N) Lg = fma(l, a.tab.WN[ix], Lg);
+            }
+            if (ghost) {
+                const double *const ew = ys < 0 ? ip.ew_lo : ip.ew_hi;
+#pragma unroll
+                for (int ix = 0; ix < Q1; ++ix) Lf = fma(lam[k][ix], ew[ix], Lf);
+                Lf = wy * fma(ys < 0 ? rw_lo : rw_hi, Lf, -Lw);
+            } else {
+#pragma unroll
+                for (int ix = 0; ix < Q1; ++ix) {
+                    const double d = DEV ? to_f64(f[k][ix]) : fma(-wy, a.tab.W[ix], to_f64(f[k][ix]));
+                    Lf = fma(lam[k][ix], d, Lf);
                 }
             }
+            const double dy = eq[2][iy][lane], L0 = Ld + Lw;
+            const double Ey = wy + dy, B = fma(drho, wy, rho * dy);
+            a0 = fma(Ey, L0, a0);
+            ax = fma(Ey, Ls, ax);
+            ay = fma(eq[3][iy][lane], L0, ay);
+            gt += fma(wy + B, Ld, fma(B, Lw, -Lf));
+            gg = fma(wy, Lg, gg);
+        }
     }
-    // gradient partials of this block, summed in a fixed order
-    red[0][threadIdx.x] = active ? -om * om * gt : 0.0;
-    red[1][threadIdx.x] = active ? gg / theta : 0.0;
-    red[2][threadIdx.x] = glo;
-    red[3][threadIdx.x] = ghi;
-    __syncthreads();
-    for (int s = ADJ_THREADS / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) {
+    if constexpr (G > 1) {
+        con[g][0][lane] = a0;
+        con[g][1][lane] = ax;
+        con[g][2][lane] = ay;
+        con[g][3][lane] = gt;
+        con[g][4][lane] = gg;
+        __syncthreads();
+        // the five sums over the groups, each by one warp
 #pragma unroll
-            for (int k = 0; k < GLBM_ADJ_NG; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + s];
+        for (int k = 0; k < 5; ++k) {
+            if (k % G != g) continue;
+            double t = con[0][k][lane];
+#pragma unroll
+            for (int u = 1; u < G; ++u) t += con[u][k][lane];
+            tot[k][lane] = t;
         }
         __syncthreads();
+        a0 = tot[0][lane];
+        ax = tot[1][lane];
+        ay = tot[2][lane];
     }
-    if (threadIdx.x == 0) {
-        const long long b = (long long)blockIdx.y * gridDim.x + blockIdx.x;
+    // mu_t = (dC/dF)^T lambda at this node (the density cancels: d f^eq_i / d f_j =
+    // E_i + sum_a dE_i/du_a (xi_j,a - u_a)), and the wall speeds' term of F_t: mu_t
+    // of every ghost this node pulls from a wall, times rho_w dE^x/du(u_w) W^y
+    double glo = 0.0, ghi = 0.0;
+    if (active) {
+        const double om = ip.omega, keep = 1.0 - om, oax = om * ax, oay = om * ay;
+        const double b0 = om * (a0 - fma(ax, ux, ay * uy));
 #pragma unroll
-        for (int k = 0; k < GLBM_ADJ_NG; ++k) a.gpart[GLBM_ADJ_NG * b + k] += red[k][0];
+        for (int k = 0; k < RPG; ++k) {
+            const int iy = g + k * G;
+            if (iy < Q1) {
+                const double b = fma(oay, f2d((float)(iy - N)), b0);
+                double *const op = a.mu_out + (iy * Q1 * plane + y * a.pitch + x);
+                const int ys = y - (iy - N);
+                const bool ghost = walls && (ys < 0 || ys >= a.Ly);
+                double gw = 0.0;
+#pragma unroll
+                for (int ix = 0; ix < Q1; ++ix) {
+                    const double m = fma(keep, lam[k][ix], ix == N ? b : fma(oax, (double)(ix - N), b));
+                    op[ix * plane] = m;
+                    if (ghost) gw = fma(m, ys < 0 ? ip.dew_lo[ix] : ip.dew_hi[ix], gw);
+                }
+                if (ghost) {
+                    gw *= a.tab.W[iy];
+                    if (ys < 0)
+                        glo = fma(gw, rw_lo, glo);
+                    else
+                        ghi = fma(gw, rw_hi, ghi);
+                }
+            }
+        }
+    }
+    // gradient partials of this block, summed in a fixed order: the groups, then
+    // the lanes
+    const bool near = walls && (y < N || y >= a.Ly - N);
+    if constexpr (G > 1) {
+        if (near) {  // (con is free: its totals are taken)
+            con[g][0][lane] = glo;
+            con[g][1][lane] = ghi;
+            __syncthreads();
+        }
+    }
+    if (g == 0) {
+        double v[GLBM_ADJ_NG] = {gt, gg, glo, ghi};
+        if constexpr (G > 1) {
+            v[0] = tot[3][lane];
+            v[1] = tot[4][lane];
+            if (near) {
+#pragma unroll
+                for (int t = 1; t < G; ++t) {
+                    v[2] += con[t][0][lane];
+                    v[3] += con[t][1][lane];
+                }
+            }
+        }
+        v[0] *= active ? -ip.omega * ip.omega : 0.0;
+        v[1] *= active ? 3.0 / N : 0.0;  // 1 / theta_x
+#pragma unroll
+        for (int k = 0; k < GLBM_ADJ_NG; ++k) {
+            if (k >= 2 && !near) continue;
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) v[k] += __shfl_down_sync(0xFFFFFFFFu, v[k], d);
+        }
+        if (lane == 0) {
+            double *const p = a.gpart + GLBM_ADJ_NG * ((long long)blockIdx.y * gridDim.x + blockIdx.x);
+            p[0] += v[0];
+            p[1] += v[1];
+            if (near) {
+                p[2] += v[2];
+                p[3] += v[3];
+            }
+        }
     }
 }
 
 // The wall speeds' term of F_T = S(X_T): mu_T = xi_x / Lx (the seed) at every
-// ghost a wall emits, times rho_w(X_T) dE^x/du(u_w) W^y, one thread per column,
-// added to the partials of the blocks of row 0 (the grid of k_adj_step's first
-// row), in a fixed order.
-template <int N, typename TF>
-__global__ void __launch_bounds__(ADJ_THREADS) k_adj_final_walls(const __grid_constant__ AdjArgs a)
+// ghost a wall emits, times rho_w(X_T) dE^x/du(u_w) W^y. The ghosts of a column
+// have sum n W^y_n = den, so the term is den / Lx sum_i xi_x,i dE^x_i/du times the
+// sum of rho_w over the columns (from k_adj_walls): one block, added to the first
+// block's partials.
+template <int N>
+__global__ void __launch_bounds__(256) k_adj_final_walls(const __grid_constant__ AdjArgs a)
 {
-    constexpr int Q1 = 2 * N + 1;
-    __shared__ double red[2][ADJ_THREADS];
-    const int x = blockIdx.x * ADJ_THREADS + threadIdx.x;
-    const InstParams &ip = *a.ip;
-    double glo = 0.0, ghi = 0.0;
-    if (x < a.Lx) {
-        const double rlo = fwd_wall_density<N, TF>(a, x, true);
-        const double rhi = fwd_wall_density<N, TF>(a, x, false);
-        for (int ny = 1; ny <= N; ++ny) {
-            const double wy = a.tab.W[N + ny];
-            for (int k = 0; k < ny; ++k)  // rows 0..ny-1 (lower), Ly-ny..Ly-1 (upper)
-                for (int ix = 0; ix < Q1; ++ix) {
-                    const double mu = (double)(ix - N) / a.Lx;
-                    glo = fma(mu * rlo * ip.dew_lo[ix], wy, glo);
-                    ghi = fma(mu * rhi * ip.dew_hi[ix], wy, ghi);
-                }
-        }
+    __shared__ double red[2][256];
+    double s[2] = {0.0, 0.0};
+    for (int x = threadIdx.x; x < a.Lx; x += 256) {
+        s[0] += a.walls[x];
+        s[1] += a.walls[a.Lx + x];
     }
-    red[0][threadIdx.x] = glo;
-    red[1][threadIdx.x] = ghi;
+    red[0][threadIdx.x] = s[0];
+    red[1][threadIdx.x] = s[1];
     __syncthreads();
-    for (int s = ADJ_THREADS / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) {
-            red[0][threadIdx.x] += red[0][threadIdx.x + s];
-            red[1][threadIdx.x] += red[1][threadIdx.x + s];
+    for (int st = 128; st > 0; st >>= 1) {
+        if ((int)threadIdx.x < st) {
+            red[0][threadIdx.x] += red[0][threadIdx.x + st];
+            red[1][threadIdx.x] += red[1][threadIdx.x + st];
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        a.gpart[GLBM_ADJ_NG * blockIdx.x + 2] += red[0][0];
-        a.gpart[GLBM_ADJ_NG * blockIdx.x + 3] += red[1][0];
+    if (threadIdx.x < 2) {
+        const double *const dew = threadIdx.x ? a.ip->dew_hi : a.ip->dew_lo;
+        double t = 0.0;
+        for (int ix = 0; ix <= 2 * N; ++ix) t = fma((double)(ix - N), dew[ix], t);
+        a.gpart[2 + threadIdx.x] += red[threadIdx.x][0] * t / (a.ip->inv_den * a.Lx);
     }
 }
 
@@ -287,50 +462,68 @@ __global__ void k_adj_seed(const __grid_constant__ AdjArgs a)
 {
     constexpr int Q1 = 2 * N + 1;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    const int q = blockIdx.z;
+    const int y = blockIdx.y, iy = blockIdx.z;
     if (x >= a.pitch) return;
-    const double v = x < a.Lx ? (double)(q % Q1 - N) / a.Lx : 0.0;
-    a.mu_out[(long long)q * a.plane + (long long)y * a.pitch + x] = v;
+    double *const p = a.mu_out + (long long)iy * Q1 * a.plane + (long long)y * a.pitch + x;
+#pragma unroll
+    for (int ix = 0; ix < Q1; ++ix)
+        p[(long long)ix * a.plane] = x < a.Lx ? (double)(ix - N) / a.Lx : 0.0;
 }
 
-__global__ void k_adj_sum(const double *gpart, long long nblocks, double *out)
+// The blocks' partials summed in a fixed order, one block.
+__global__ void __launch_bounds__(256) k_adj_sum(const double *gpart, long long nblocks, double *out)
 {
-    if (threadIdx.x < GLBM_ADJ_NG) {
-        double s = 0.0;
-        for (long long b = 0; b < nblocks; ++b) s += gpart[GLBM_ADJ_NG * b + threadIdx.x];
-        out[threadIdx.x] = s;
+    __shared__ double red[256];
+    const int k = threadIdx.x % GLBM_ADJ_NG;
+    double s = 0.0;
+    for (long long b = threadIdx.x / GLBM_ADJ_NG; b < nblocks; b += 256 / GLBM_ADJ_NG)
+        s += gpart[GLBM_ADJ_NG * b + k];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int st = 128; st >= GLBM_ADJ_NG; st >>= 1) {
+        if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
+        __syncthreads();
     }
+    if (threadIdx.x < GLBM_ADJ_NG) out[threadIdx.x] = red[threadIdx.x];
+}
+
+// The wall sums of a (a.mu_in, a.X).
+template <int N>
+cudaError_t adj_walls_n(const AdjArgs &a, int quantities, cudaStream_t s)
+{
+    const dim3 grid((a.Lx + ADJ_WX - 1) / ADJ_WX, quantities);
+    return a.prec == GLBM_FP64
+               ? launch_serialized(k_adj_walls<N, double>, grid, dim3(ADJ_WX * ADJ_WS), s, a)
+               : launch_serialized(k_adj_walls<N, float>, grid, dim3(ADJ_WX * ADJ_WS), s, a);
 }
 
 template <int N>
 cudaError_t adj_step_n(const AdjArgs &a, cudaStream_t s)
 {
-    k_adj_wall<N><<<(a.Lx + 63) / 64, 64, 0, s>>>(a);
-    dim3 grid((a.Lx + ADJ_THREADS - 1) / ADJ_THREADS, a.Ly);
-    if (a.prec == GLBM_FP64)
-        k_adj_step<N, double><<<grid, ADJ_THREADS, 0, s>>>(a);
-    else
-        k_adj_step<N, float><<<grid, ADJ_THREADS, 0, s>>>(a);
-    return cudaGetLastError();
+    if (a.bc == GLBM_BC_WALLS) {
+        const cudaError_t e = adj_walls_n<N>(a, 4, s);
+        if (e != cudaSuccess) return e;
+    }
+    const dim3 grid((a.Lx + 31) / 32, a.Ly);
+    return a.prec == GLBM_FP64
+               ? launch_serialized(k_adj_step<N, double>, grid, dim3(32 * ADJ_G<N>), s, a)
+               : launch_serialized(k_adj_step<N, float>, grid, dim3(32 * ADJ_G<N>), s, a);
 }
 
 template <int N>
 cudaError_t adj_final_walls_n(const AdjArgs &a, cudaStream_t s)
 {
     if (a.bc != GLBM_BC_WALLS) return cudaSuccess;
-    const int blocks = (a.Lx + ADJ_THREADS - 1) / ADJ_THREADS;
-    if (a.prec == GLBM_FP64)
-        k_adj_final_walls<N, double><<<blocks, ADJ_THREADS, 0, s>>>(a);
-    else
-        k_adj_final_walls<N, float><<<blocks, ADJ_THREADS, 0, s>>>(a);
+    const cudaError_t e = adj_walls_n<N>(a, 2, s);
+    if (e != cudaSuccess) return e;
+    k_adj_final_walls<N><<<1, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 template <int N>
 cudaError_t adj_seed_n(const AdjArgs &a, cudaStream_t s)
 {
-    dim3 grid((a.pitch + 127) / 128, a.Ly, (2 * N + 1) * (2 * N + 1));
+    dim3 grid((a.pitch + 127) / 128, a.Ly, 2 * N + 1);
     k_adj_seed<N><<<grid, 128, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -339,7 +532,7 @@ cudaError_t adj_seed_n(const AdjArgs &a, cudaStream_t s)
 
 long long glbm_adj_blocks(int Lx, int Ly)
 {
-    return (long long)((Lx + ADJ_THREADS - 1) / ADJ_THREADS) * Ly;
+    return (long long)((Lx + 31) / 32) * Ly;
 }
 
 cudaError_t glbm_launch_adj_seed(const AdjArgs &a, cudaStream_t s)
@@ -380,6 +573,6 @@ cudaError_t glbm_launch_adj_step(const AdjArgs &a, cudaStream_t s)
 
 cudaError_t glbm_launch_adj_sum(const double *gpart, long long nblocks, double *out, cudaStream_t s)
 {
-    k_adj_sum<<<1, 32, 0, s>>>(gpart, nblocks, out);
+    k_adj_sum<<<1, 256, 0, s>>>(gpart, nblocks, out);
     return cudaGetLastError();
 }

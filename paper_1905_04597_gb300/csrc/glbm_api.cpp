@@ -1517,6 +1517,33 @@ static cudaError_t launch_2d_between(const glbm_ctx *c, const void *fin, void *f
                                 : glbm_launch_step2d_f32(N, c->tile[N], a, c->n_inst, s);
 }
 
+// Advance len steps from the current state X_t with X_t .. X_{t+len-1} left in
+// `states` (len state copies) and X_{t+len} as the new current state. *done is
+// false, and the state X_t again, if a node left the positivity domain: the
+// caller's glbm_step then stops at the failing step.
+static glbm_status step_into(glbm_ctx *c, int64_t len, char *states, bool *done)
+{
+    const size_t pool = bytes_state(c);
+    const int64_t t0 = c->t;
+    CUDA_TRY(cudaMemcpyAsync(states, c->buf[c->cur], pool, cudaMemcpyDeviceToDevice, c->stream));
+    for (int64_t r = 0; r < len; ++r) {
+        void *out = r + 1 < len ? states + pool * (r + 1) : c->buf[1 - c->cur];
+        CUDA_TRY(launch_2d_between(c, states + pool * r, out, c->stream));
+        c->launches += launches_per_step(c);
+    }
+    glbm_status st = read_status(c);
+    if (st != GLBM_OK) return st;
+    *done = (c->h_status[ST_FLAGS] & ST_UNSTABLE) == 0u;
+    if (*done) {
+        c->cur = 1 - c->cur;
+        c->t = t0 + len;
+        return GLBM_OK;
+    }
+    CUDA_TRY(set_clock(c, t0));
+    CUDA_TRY(clear_unstable(c));
+    return GLBM_OK;
+}
+
 struct Scratch {
     const DevAlloc &A;
     cudaStream_t s;
@@ -1556,19 +1583,26 @@ extern "C" glbm_status glbm_adjoint_flowrate(glbm_ctx *c, int64_t steps, int64_t
     char *ck = (char *)S.get(pool * nseg);
     char *seg = (char *)S.get(pool * K);
     double *mu0 = (double *)S.get(mu_bytes), *mu1 = (double *)S.get(mu_bytes);
-    double *G = (double *)S.get(2 * (size_t)g.Lx * sizeof(double));
+    double *wsum = (double *)S.get(4 * (size_t)g.Lx * sizeof(double));
     double *gpart = (double *)S.get(GLBM_ADJ_NG * (size_t)nblk * sizeof(double));
     double *gsum = (double *)S.get(GLBM_ADJ_NG * sizeof(double));
-    if (!ck || !seg || !mu0 || !mu1 || !G || !gpart || !gsum)
+    if (!ck || !seg || !mu0 || !mu1 || !wsum || !gpart || !gsum)
         return fail(GLBM_E_NOMEM, "adjoint scratch of %.1f MB failed",
                     (pool * (nseg + K) + 2.0 * mu_bytes) / 1e6);
     const int64_t t_start = c->t;
 
-    // forward with checkpoints
+    // forward with checkpoints; the last segment's steps go through the segment
+    // buffer, where the backward sweep needs their states first (no recompute)
+    bool seg_filled = false;
     for (int64_t s = 0; s < nseg; ++s) {
         CUDA_TRY(cudaMemcpyAsync(ck + pool * s, c->buf[c->cur], pool, cudaMemcpyDeviceToDevice, c->stream));
         const int64_t len = std::min<int64_t>(K, steps - s * K);
-        glbm_status st = glbm_step(c, len);
+        glbm_status st = GLBM_OK;
+        if (s == nseg - 1 && !c->halted) {
+            st = step_into(c, len, seg, &seg_filled);
+            if (st != GLBM_OK) return st;
+        }
+        if (!seg_filled) st = glbm_step(c, len);
         if (st != GLBM_OK) return st;
     }
     for (int i = 0; i < c->n_inst; ++i) {
@@ -1585,8 +1619,7 @@ extern "C" glbm_status glbm_adjoint_flowrate(glbm_ctx *c, int64_t steps, int64_t
         memset(&a, 0, sizeof(a));
         a.tab = glbm_narrow_table(c->tabs[g.N]);
         a.ip = c->d_ip + i;
-        a.G = G;
-        a.Gw = G;
+        a.walls = wsum;
         a.gpart = gpart;
         a.Lx = g.Lx;
         a.Ly = g.Ly;
@@ -1604,12 +1637,15 @@ extern "C" glbm_status glbm_adjoint_flowrate(glbm_ctx *c, int64_t steps, int64_t
         CUDA_TRY(glbm_launch_adj_final_walls(a, c->stream));
         for (int64_t s = nseg - 1; s >= 0; --s) {
             const int64_t t0 = s * K, len = std::min<int64_t>(K, steps - t0);
-            // recompute X_t0 .. X_t0+len-1 with the dither counter of the forward pass
-            CUDA_TRY(cudaMemcpyAsync(seg, ck + pool * s, pool, cudaMemcpyDeviceToDevice, c->stream));
-            CUDA_TRY(set_clock(c, t_start + t0));
-            for (int64_t r = 0; r + 1 < len; ++r) {
-                CUDA_TRY(launch_2d_between(c, seg + pool * r, seg + pool * (r + 1), c->stream));
-                c->launches += launches_per_step(c);
+            // recompute X_t0 .. X_t0+len-1 with the dither counter of the forward
+            // pass, unless the segment buffer still holds them
+            if (!seg_filled || s < nseg - 1 || (i > 0 && nseg > 1)) {
+                CUDA_TRY(cudaMemcpyAsync(seg, ck + pool * s, pool, cudaMemcpyDeviceToDevice, c->stream));
+                CUDA_TRY(set_clock(c, t_start + t0));
+                for (int64_t r = 0; r + 1 < len; ++r) {
+                    CUDA_TRY(launch_2d_between(c, seg + pool * r, seg + pool * (r + 1), c->stream));
+                    c->launches += launches_per_step(c);
+                }
             }
             for (int64_t r = len - 1; r >= 0; --r) {
                 a.X = seg + pool * r + (size_t)c->geo[i].off * c->elem;

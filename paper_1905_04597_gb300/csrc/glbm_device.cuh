@@ -440,6 +440,9 @@ __device__ __forceinline__ double f2d(float x)
     return e ? __hiloint2double((int)hi, (int)(b << 29)) : 0.0;
 }
 
+__device__ __forceinline__ double to_f64(float x) { return f2d(x); }
+__device__ __forceinline__ double to_f64(double x) { return x; }
+
 // Knuth's two-sum on both lanes (the packed form of acc2).
 __device__ __forceinline__ void acc2x2(f32x2 &s, f32x2 &c, f32x2 x)
 {
@@ -480,4 +483,34 @@ __device__ __forceinline__ int wrap_shift(int i, int L, bool one_wrap)
 {
     if (one_wrap) return i < 0 ? i + L : (i >= L ? i - L : i);
     return wrap_index(i, L);
+}
+
+// Launch with programmatic stream serialization (see wait_prior_grid), except
+// the first step of a dataflow chunk, which waits for all work before it.
+template <class TY>
+inline bool programmatic(const Step2DArgsT<TY> &a)
+{
+    return !(a.bands && a.node == 0);
+}
+template <typename Args>
+inline bool programmatic(const Args &)
+{
+    return true;
+}
+
+template <typename Args>
+inline cudaError_t launch_serialized(void (*kern)(Args), dim3 grid, dim3 block, cudaStream_t s,
+                                     const Args &a)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = 0;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = programmatic(a) ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, a);
 }

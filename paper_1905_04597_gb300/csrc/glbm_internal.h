@@ -335,8 +335,8 @@ struct AdjArgs {
     const void *X;         // forward state X_t of the instance (FP64, or FP32 deviations)
     const double *mu_in;   // mu_{t+1} = dJ/dF_{t+1}, pitched like the populations
     double *mu_out;        // mu_t
-    const double *G;       // [2][Lx] wall sums of mu_in (lower, upper)
-    double *Gw;            // the same array, written by the wall kernel
+    double *walls;         // [4][Lx]: rho_w of X (lower, upper wall), and the wall sums of
+                           // mu_in over den, written before each step
     double *gpart;         // [blocks][GLBM_ADJ_NG] partials of dJ/dtau, dJ/dg, dJ/du_lo,
                            // dJ/du_hi, summed over steps
     int Lx, Ly, pitch, bc, N, prec;

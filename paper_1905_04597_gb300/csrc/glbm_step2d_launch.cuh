@@ -46,36 +46,6 @@ __global__ void __launch_bounds__(32 * G * R)
     }
 }
 
-// Launch with programmatic stream serialization (see wait_prior_grid), except
-// the first step of a dataflow chunk, which waits for all work before it.
-template <class TY>
-inline bool programmatic(const Step2DArgsT<TY> &a)
-{
-    return !(a.bands && a.node == 0);
-}
-template <typename Args>
-inline bool programmatic(const Args &)
-{
-    return true;
-}
-
-template <typename Args>
-inline cudaError_t launch_serialized(void (*kern)(Args), dim3 grid, dim3 block, cudaStream_t s,
-                                     const Args &a)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = programmatic(a) ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, a);
-}
-
 // The wall-density launch that precedes a step whose arguments carry a
 // wall-density buffer (Step2DArgs::rw); nothing otherwise.
 template <int N, typename T, int NXL, int ZY, int ZX, class Args>
