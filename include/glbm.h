@@ -396,6 +396,11 @@ glbm_status glbm_adjoint_flowrate(glbm_ctx *ctx, int64_t steps, int64_t ckpt_eve
  * packed two-lane arithmetic), and each node's 2k+3 velocity rows are dealt
  * to G warps. Every level k (0..GLBM_LEVELS-1) and precision has up to
  * GLBM_MAX_TILES candidate shapes; entry 0 is the default of a new context.
+ * New uniform FP64 contexts of small lattices with the linearised force step with
+ * a kernel of their own instead (one thread per node and velocity row, the
+ * results those of entry 0 bit for bit; no dataflow chunks and no wall-density
+ * launch); glbm_set_tiles of their level, glbm_set_wall_launch(0 or 1) and
+ * glbm_set_dataflow take the tiles from then on, glbm_autotune keeps the faster.
  *
  * glbm_tile_count returns the number of candidates of level k in precision
  * prec (0 for an invalid pair); glbm_tile_shape returns candidate idx. Both

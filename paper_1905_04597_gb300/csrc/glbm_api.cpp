@@ -139,6 +139,8 @@ struct glbm_ctx {
     int n_items = 0;
     int group[GLBM_MAXN + 2] = {0};  // first item of each level
     int tile[GLBM_MAXN + 1] = {0};   // tile shape index per level (glbm_tiles.h)
+    bool small = false;              // steps with glbm_step2d_small.cuh
+    AxisTableHi *d_tabs = nullptr;   // the axes' tables (y, x) of a small context
     std::vector<ChunkGraph> graphs;  // captured chunks, by their buffers and form
     int dataflow = 1;              // 1: dataflow chunks where the context allows them
     unsigned *d_df = nullptr;      // per-step CTA counts of a chunk, then the band counts
@@ -388,6 +390,7 @@ static void destroy_resources(glbm_ctx *c)
     dev_free(c->A, c->d_stage, c->stream);
     dev_free(c->A, c->d_items, c->stream);
     dev_free(c->A, c->d_rw, c->stream);
+    dev_free(c->A, c->d_tabs, c->stream);
     if (c->h_status) cudaFreeHost(c->h_status);
     if (c->cap) cudaStreamDestroy(c->cap);
 }
@@ -575,6 +578,8 @@ static glbm_status finish_create(glbm_ctx *c, const glbm_config *cfgs, int n, vo
     return GLBM_OK;
 }
 
+static glbm_status choose_small(glbm_ctx *c);
+
 extern "C" glbm_status glbm_create(const glbm_config *cfgs, int n, void *stream, glbm_ctx **out)
 {
     if (!cfgs || n < 1 || !out) return fail(GLBM_E_INVAL, "null argument or n < 1");
@@ -596,6 +601,7 @@ extern "C" glbm_status glbm_create(const glbm_config *cfgs, int n, void *stream,
     glbm_ctx *c = new (std::nothrow) glbm_ctx();
     if (!c) return fail(GLBM_E_NOMEM, "host allocation failed");
     glbm_status st = finish_create(c, cfgs, n, stream);
+    if (st == GLBM_OK) st = choose_small(c);
     if (st != GLBM_OK) {
         destroy_resources(c);
         delete c;
@@ -628,6 +634,34 @@ static int ctx_tile_shapes(const glbm_ctx *c, int N, TileShape *out)
     if (c->dims == 3) return glbm_tile_shapes_3d(N, c->prec, out);
     if (is_zv(c)) return glbm_tile_shapes_zv(N, zv_kind(c), c->prec, out);
     return is_x1(c) ? glbm_tile_shapes_x1(N, c->prec, out) : glbm_tile_shapes(N, c->prec, out);
+}
+
+// Whether a new context's FP64 steps take glbm_step2d_small.cuh: uniform 2D
+// lattices with the linearised force whose (node, velocity row) threads make at
+// most SMALL_WARPS warps (three per SM sub-partition), and more by the factor that
+// the tiles' 32-column rows waste on a lattice narrower than 16 columns. Measured
+// (GB300, D2Q81 unless noted, us per step, tiles -> small): 40 x 24 (270 warps)
+// 20.4 -> 8.6, 64 x 64 (1152) 20.3 -> 14.6, 128 x 64 (2304) 20.4 -> 24.3, 8 x 100
+// 22.1 -> 8.2; D2Q289 4 x 60 44.4 -> 17.4; D1Q3 x D1Q28 5 instances of 1 x 200 106.6
+// -> 14.0. Choosing a tile shape, a wall-density mode or a dataflow mode afterwards
+// takes the tiles (the results are the same).
+static const long long SMALL_WARPS = 3 * 608;
+static glbm_status choose_small(glbm_ctx *c)
+{
+    if (c->dims != 2 || c->hetero || c->prec != GLBM_FP64 || is_guo(c)) return GLBM_OK;
+    const Geo &g = c->geo[0];
+    const long long rows = 2 * g.N + 1 + ((g.zv & GLBM_ZV_Y) ? 1 : 0);
+    const long long waste = g.Lx < 16 ? 16 / g.Lx : 1;
+    if (c->n_inst > 65535 || c->n_inst * g.nodes() * rows > 32 * SMALL_WARPS * waste) return GLBM_OK;
+    c->d_tabs = (AxisTableHi *)dev_alloc(c->A, 2 * sizeof(AxisTableHi), c->stream);
+    if (!c->d_tabs) return fail(GLBM_E_NOMEM, "device allocation of the axis tables failed");
+    const AxisTableHi *src[2] = {&tab_y(c, g), &tab_x(c, g)};
+    for (int i = 0; i < 2; ++i)
+        CUDA_TRY(cudaMemcpyAsync(c->d_tabs + i, src[i], sizeof(AxisTableHi), cudaMemcpyHostToDevice,
+                                 c->stream));
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    c->small = true;
+    return GLBM_OK;
 }
 
 static TileShape tile_of(const glbm_ctx *c, int N)
@@ -960,9 +994,29 @@ static BatchArgs batch_args(const glbm_ctx *c, int from)
     return batch_args(c, c->buf[from], c->buf[1 - from]);
 }
 
+static cudaError_t launch_small(const glbm_ctx *c, const void *fin, void *fout, cudaStream_t s)
+{
+    const Geo &g = c->geo[0];
+    SmallArgs a;
+    a.ty = c->d_tabs;
+    a.tx = c->d_tabs + 1;
+    a.fin = static_cast<const double *>(fin);
+    a.fout = static_cast<double *>(fout);
+    a.ip = c->d_ip;
+    a.status = c->d_status;
+    a.Lx = g.Lx;
+    a.Ly = g.Ly;
+    a.pitch = g.pitch;
+    a.bc = c->cfg[0].bc;
+    a.plane = (int)g.plane;
+    a.inst_stride = c->n_inst > 1 ? c->geo[1].off : 0;
+    return glbm_launch_step2d_small(g.N, g.NX, g.zv, a, c->n_inst, s);
+}
+
 // Kernel launches of one 2D step.
 static int launches_per_step(const glbm_ctx *c)
 {
+    if (c->small) return 1;
     return c->hetero ? glbm_batched_launches(batch_args(c, 0)) : (c->wall_launch ? 2 : 1);
 }
 
@@ -972,7 +1026,7 @@ static int launches_per_step(const glbm_ctx *c)
 static bool df_eligible(const glbm_ctx *c)
 {
     return c->dataflow && !c->hetero && c->dims == 2 && c->geo[0].N <= GLBM_MAXN_2N1 &&
-           !c->wall_launch;
+           !c->wall_launch && !c->small;
 }
 
 // One 2D (or 3D) step of every instance from state buffer fin into fout, on
@@ -982,6 +1036,7 @@ static cudaError_t launch_step(const glbm_ctx *c, const void *fin, void *fout, c
 {
     if (c->hetero) return glbm_launch_batched_f32(batch_args(c, fin, fout), s);
     const int N = c->geo[0].N;
+    if (c->small) return launch_small(c, fin, fout, s);
     if (c->dims == 3)
         return glbm_launch_step3d(N, c->prec, c->tile[N], step3d_args(c, fin, fout), c->n_inst, s);
     if (N > GLBM_MAXN_2N1)
@@ -1507,6 +1562,7 @@ static cudaError_t launch_2d_between(const glbm_ctx *c, const void *fin, void *f
 {
     const int N = c->geo[0].N;
     if (N > GLBM_MAXN_2N1) return cudaErrorInvalidValue;  // the adjoint takes levels <= 8
+    if (c->small) return launch_small(c, fin, fout, s);
     Step2DArgs a = step_args(c, 0);
     a.fin = fin;
     a.fout = fout;
@@ -1723,8 +1779,9 @@ extern "C" glbm_status glbm_set_dataflow(glbm_ctx *c, int on)
 {
     if (!c) return fail(GLBM_E_INVAL, "null context");
     if (on < 0 || on > 2) return fail(GLBM_E_INVAL, "dataflow mode %d (0, 1 or 2)", on);
-    const bool changed = on != c->dataflow;
+    const bool changed = on != c->dataflow || c->small;
     c->dataflow = on;
+    c->small = false;
     return changed ? tiles_changed(c) : GLBM_OK;  // the chunk graphs carry the mode
 }
 
@@ -1745,6 +1802,7 @@ extern "C" glbm_status glbm_set_wall_launch(glbm_ctx *c, int mode)
         if (st != GLBM_OK) return st;
     }
     c->wall_launch = on;
+    if (mode >= 0) c->small = false;
     return tiles_changed(c);  // the captured step graphs name the old launches
 }
 
@@ -1764,8 +1822,11 @@ extern "C" glbm_status glbm_set_tiles(glbm_ctx *c, const int *tiles)
         if (tiles[k] < -1 || tiles[k] >= (n > 0 ? n : 1))
             return fail(GLBM_E_INVAL, "tile index %d out of range for k=%d", tiles[k], k);
     }
-    for (int k = 0; k < GLBM_LEVELS; ++k)
-        if (tiles[k] >= 0) c->tile[k + 1] = tiles[k];
+    for (int k = 0; k < GLBM_LEVELS; ++k) {
+        if (tiles[k] < 0) continue;
+        c->tile[k + 1] = tiles[k];
+        if (c->geo[0].N == k + 1) c->small = false;
+    }
     return tiles_changed(c);
 }
 
@@ -1871,6 +1932,8 @@ extern "C" glbm_status glbm_autotune(glbm_ctx *c, int reps, double *us)
     CUDA_TRY(cudaEventCreate(&e0));
     cudaError_t ce = cudaEventCreate(&e1);
     glbm_status st = ce == cudaSuccess ? GLBM_OK : fail(GLBM_E_CUDA, "event: %s", cudaGetErrorString(ce));
+    const bool small0 = c->small;  // timed against the tuned tiles at the end
+    c->small = false;
     for (int N = 1; N <= GLBM_MAXN && st == GLBM_OK; ++N) {
         if (!level_present(c, N)) continue;
         TileShape sh[GLBM_MAX_TILES];
@@ -1922,6 +1985,19 @@ extern "C" glbm_status glbm_autotune(glbm_ctx *c, int reps, double *us)
     if (st == GLBM_OK && !c->hetero && c->dims == 2 && c->geo[0].N <= GLBM_MAXN_2N1) {
         c->dataflow = 1;
         st = autotune_dataflow(c, e0, e1);
+    }
+    if (small0) {
+        glbm_status sp = spare_ready(c);  // (time_steps runs through three buffers)
+        c->small = sp != GLBM_OK;
+        if (st == GLBM_OK && sp == GLBM_OK) {
+            float ms[2] = {0.f, 0.f};
+            for (int m = 0; m < 2 && st == GLBM_OK; ++m) {
+                c->small = m == 1;
+                st = tiles_changed(c);
+                if (st == GLBM_OK) st = time_steps(c, 2 * kGraphChunk, df_eligible(c), e0, e1, &ms[m]);
+            }
+            c->small = ms[1] < ms[0];
+        }
     }
     if (e1) cudaEventDestroy(e1);
     cudaEventDestroy(e0);

@@ -261,6 +261,22 @@ template <int N, typename T>
 cudaError_t glbm_step2d_zv_level(int kind, int shape, const Step2DArgsOf<N> &a, int n_inst,
                                  cudaStream_t s);
 
+// The FP64 step of small 2D lattices (glbm_step2d_small.cuh).
+struct SmallArgs {
+    const AxisTableHi *ty, *tx;  // device copies of the axes' tables
+    const double *fin;
+    double *fout;
+    const InstParams *ip;
+    unsigned *status;
+    int Lx, Ly, pitch, bc;
+    int plane;                   // elements per velocity plane (Q plane < 2^31)
+    long long inst_stride;
+};
+cudaError_t glbm_launch_step2d_small(int N, int NX, int zv, const SmallArgs &a, int n_inst,
+                                     cudaStream_t s);
+cudaError_t glbm_launch_step2d_small_zv(int N, int zv, const SmallArgs &a, int n_inst,
+                                        cudaStream_t s);
+
 // 3D tensor products (glbm_step3d.cu): levels 1..3, isotropic, periodic in x
 // and z, walls or periodicity in y.
 struct Step3DArgs {

@@ -37,7 +37,9 @@ struct Step2D {
     static constexpr int RPG = (Q1 + G - 1) / G;  // velocity rows per warp group
     static constexpr int NW = G * R;              // warps per CTA
     static constexpr int NT = 32 * NW;
-    static constexpr int NV = 4;                  // wall-flux accumulators
+    // wall-flux accumulators: an FP64 addition depends on the one before it for 64
+    // cycles, so FP64 takes more of them where four would add more than 64 values each
+    static constexpr int NV = sizeof(T) == 8 && AY::NPAIR * QX > 256 ? 16 : 4;
     static constexpr bool DX_SHARED = G > 1 && sizeof(T) == 4;  // E^x - W read from smem
     static constexpr bool DEV = sizeof(T) == 4;   // FP32 deviation storage
     using A = TabAcc<T>;
@@ -110,18 +112,16 @@ struct Step2D {
             dsum[v][1][lane] = shi;
         }
         __syncthreads();
-        if (w == 0) {
-            T s0 = T(0), s1 = T(0);
 #pragma unroll
-            for (int j = 0; j < NV; ++j) {
-                s0 += dsum[j][0][lane];
-                s1 += dsum[j][1][lane];
-            }
+        for (int h = 0; h < 2; ++h) {
+            if (w != (nw > 1 ? h : 0)) continue;
+            T s0 = T(0);
+#pragma unroll
+            for (int j = 0; j < NV; ++j) s0 += dsum[j][h][lane];
             const T inv_den = DEV ? (T)ip.inv_den_f : (T)ip.inv_den;
             // FP64: rho_w = D / den.  FP32: rho_w - 1 = (D - den) / den, and
             // D - den is the sum of the absorbed deviations.
-            rw[0][lane] = s0 * inv_den;
-            rw[1][lane] = s1 * inv_den;
+            rw[h][lane] = s0 * inv_den;
         }
         __syncthreads();
     }
