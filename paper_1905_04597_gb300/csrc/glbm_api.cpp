@@ -558,20 +558,9 @@ static glbm_status finish_create(glbm_ctx *c, const glbm_config *cfgs, int n, vo
     // rest state X = W everywhere
     glbm_status st = ensure_stage(c, 4 * (size_t)max_nodes);
     if (st != GLBM_OK) return st;
-    std::vector<double> one(max_nodes, 1.0), zero(max_nodes, 0.0);
-    CUDA_TRY(cudaMemcpy(c->d_stage, one.data(), max_nodes * 8, cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(c->d_stage + max_nodes, zero.data(), max_nodes * 8, cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(c->d_stage + 2 * max_nodes, zero.data(), max_nodes * 8, cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(c->d_stage + 3 * max_nodes, zero.data(), max_nodes * 8, cudaMemcpyHostToDevice));
     for (int i = 0; i < n; ++i) {
-        if (c->dims == 3)
-            CUDA_TRY(glbm_launch_set_equilibrium3d(aux_args(c, i), inst_ptr(c, 0, i), 0, c->d_stage,
-                                                   c->d_stage + max_nodes, c->d_stage + 2 * max_nodes,
-                                                   c->d_stage + 3 * max_nodes, c->stream));
-        else
-            CUDA_TRY(glbm_launch_set_equilibrium(aux_args(c, i), inst_ptr(c, 0, i), 0, c->d_stage,
-                                                 c->d_stage + max_nodes, c->d_stage + 2 * max_nodes,
-                                                 c->stream));
+        CUDA_TRY(glbm_launch_set_equilibrium(aux_args(c, i), inst_ptr(c, 0, i), nullptr, nullptr,
+                                             nullptr, nullptr, c->stream));
         c->launches += 1;
     }
     CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -776,7 +765,7 @@ static glbm_status set_equilibrium_impl(glbm_ctx *c, int inst, const double *rho
     if (!rho || !ux || (c->dims >= 2 && !uy)) return fail(GLBM_E_INVAL, "null field");
     const size_t nodes = (size_t)c->geo[inst].nodes();
     const double *dr = rho, *du = ux, *dv = uy, *dw = uz;
-    if (!on_device || (c->dims == 3 && !uz)) {
+    if (!on_device) {
         st = ensure_stage(c, 4 * nodes);
         if (st != GLBM_OK) return st;
     }
@@ -789,21 +778,11 @@ static glbm_status set_equilibrium_impl(glbm_ctx *c, int inst, const double *rho
             CUDA_TRY(cudaMemcpyAsync(c->d_stage + 3 * nodes, uz, nodes * 8, cudaMemcpyHostToDevice, c->stream));
         dr = c->d_stage;
         du = c->d_stage + nodes;
-        dv = c->dims >= 2 ? c->d_stage + 2 * nodes : c->d_stage;
+        dv = c->d_stage + 2 * nodes;
         if (uz) dw = c->d_stage + 3 * nodes;
     }
-    if (!dv) dv = du;
-    if (c->dims == 3) {
-        if (!dw) {  // u_z = 0
-            CUDA_TRY(cudaMemsetAsync(c->d_stage + 3 * nodes, 0, nodes * 8, c->stream));
-            dw = c->d_stage + 3 * nodes;
-        }
-        CUDA_TRY(glbm_launch_set_equilibrium3d(aux_args(c, inst), inst_ptr(c, c->cur, inst), 0, dr, du,
-                                               dv, dw, c->stream));
-    } else {
-        CUDA_TRY(glbm_launch_set_equilibrium(aux_args(c, inst), inst_ptr(c, c->cur, inst), 0, dr, du,
-                                             dv, c->stream));
-    }
+    CUDA_TRY(glbm_launch_set_equilibrium(aux_args(c, inst), inst_ptr(c, c->cur, inst), dr, du, dv, dw,
+                                         c->stream));
     c->launches += 1;
     CUDA_TRY(set_clock(c, 0));
     CUDA_TRY(clear_unstable(c));

@@ -1,5 +1,4 @@
-// Auxiliary kernels of libglbm: initial equilibrium, import/export of
-// populations in the FP64 logical layout, the 1D moment reducer (2D and 3D:
+// Auxiliary kernels of libglbm: import/export of populations in the FP64 logical layout, the 1D moment reducer (2D and 3D:
 // glbm_moments.cuh), deterministic global sums, and the 1D step (Sec. 5.1 shock
 // tube, halfway bounce-back) both per launch and resident in one CTA for many
 // steps.
@@ -9,47 +8,6 @@
 #include "glbm_device.cuh"
 
 namespace {
-
-// E_i(u) - W_i of velocity index i at runtime level t.N (FP64 Horner on the
-// coefficient table; on the 2N+2 hierarchy the velocity is +-(2m+1)).
-__device__ double eq_dev_rt(const AxisTableHi &t, double u, int i)
-{
-    const int N = t.N;
-    const int n = ax_vel(t, i);
-    const int an = n < 0 ? -n : n;
-    const int m = t.zv ? (an - 1) / 2 : an;
-    const double v = u * u;
-    double ae = t.Ce[m][N];
-    for (int k = N - 1; k >= 1; --k) ae = fma(ae, v, t.Ce[m][k]);
-    ae *= v;
-    double bo = 0.0;
-    if (an > 0) {
-        bo = t.Co[m][N - 1];
-        for (int k = N - 2; k >= 0; --k) bo = fma(bo, v, t.Co[m][k]);
-    }
-    return n >= 0 ? fma(u, bo, ae) : fma(-u, bo, ae);
-}
-
-// E_i(u) - W_i of every velocity index of a runtime level, the mirror pairs
-// (i, Q - 1 - i), whose velocities are opposite, from one evaluation of the
-// even and odd parts each: the same operations as eq_dev_rt per index.
-__device__ void eq_dev_all_rt(const AxisTableHi &t, double u, double *out)
-{
-    const int N = t.N, Q = ax_q(t);
-    const double v = u * u;
-    for (int p = 0; p < Q / 2; ++p) {
-        const int an = ax_vel(t, Q - 1 - p);  // > 0
-        const int m = t.zv ? (an - 1) / 2 : an;
-        double ae = t.Ce[m][N];
-        for (int k = N - 1; k >= 1; --k) ae = fma(ae, v, t.Ce[m][k]);
-        ae *= v;
-        double bo = t.Co[m][N - 1];
-        for (int k = N - 2; k >= 0; --k) bo = fma(bo, v, t.Co[m][k]);
-        out[Q - 1 - p] = fma(u, bo, ae);
-        out[p] = fma(-u, bo, ae);
-    }
-    if (Q & 1) out[Q / 2] = eq_dev_rt(t, u, Q / 2);
-}
 
 __device__ __forceinline__ double load_full(const AuxArgs &a, const void *f, long long idx, int q)
 {
@@ -68,48 +26,6 @@ __device__ __forceinline__ double rest_weight(const AuxArgs &a, int q)
     }
     const int Qx = ax_q(a.tabx);
     return a.tab.W[q / Qx] * a.tabx.W[q % Qx];
-}
-
-__global__ void k_set_equilibrium(const __grid_constant__ AuxArgs a, void *f, int inst,
-                                  const double *__restrict__ rho, const double *__restrict__ ux,
-                                  const double *__restrict__ uy)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= a.Lx) return;
-    // 1D: the only axis is x, with table tab and level N
-    const AxisTableHi &tx = a.dims == 2 ? a.tabx : a.tab;
-    const int Q1x = ax_q(tx);
-    const long long node = (long long)y * a.Lx + x;
-    const double r = rho[node], u = ux[node], v = a.dims == 2 ? uy[node] : 0.0;
-    const long long base = (long long)inst * a.inst_stride + (long long)y * a.pitch + x;
-    const int Qy = a.dims == 2 ? ax_q(a.tab) : 1;
-    const bool f64 = a.prec == GLBM_FP64;
-    double exs[GLBM_MAXQA];  // per node: E^x (FP64 storage) or E^x - W^x (FP32 deviations)
-    double dys[GLBM_MAXQA];  // E^y - W^y
-    eq_dev_all_rt(tx, u, exs);
-    if (f64)
-        for (int ix = 0; ix < Q1x; ++ix) exs[ix] += tx.W[ix];
-    if (a.dims == 2) eq_dev_all_rt(a.tab, v, dys);
-    for (int iy = 0; iy < Qy; ++iy) {
-        const double wy = a.dims == 2 ? a.tab.W[iy] : 1.0;
-        const double dy = a.dims == 2 ? dys[iy] : 0.0;
-        // per row: A = rho E^y and B = rho E^y - W^y = (rho - 1) W^y + rho d^y
-        // (no cancellation); then rho E^x E^y = E^x A and, in deviations,
-        // rho E^x E^y - W^x W^y = W^x B + d^x A: one or two FP64 operations
-        // per population
-        const double A = r * (wy + dy);
-        const double B = fma(r - 1.0, wy, r * dy);
-        const long long row = base + (long long)(iy * Q1x) * a.plane;
-        if (f64) {
-            double *out = static_cast<double *>(f) + row;
-            for (int ix = 0; ix < Q1x; ++ix) out[(long long)ix * a.plane] = exs[ix] * A;
-        } else {
-            float *out = static_cast<float *>(f) + row;
-            for (int ix = 0; ix < Q1x; ++ix)
-                out[(long long)ix * a.plane] = (float)fma(exs[ix], A, tx.W[ix] * B);
-        }
-    }
 }
 
 __global__ void k_set_populations(const __grid_constant__ AuxArgs a, void *f, int inst,
@@ -470,69 +386,7 @@ cudaError_t launch_resident_t(const AuxArgs &a, void *fv, int inst, long long st
     }
 }
 
-// ---------------------------------------------------------------------------
-// 3D tensor products: level N on every axis, layout f[q][z][y][x] with
-// q = (iz Q1 + iy) Q1 + ix, periodic in x and z, walls or periodicity in y.
-// ---------------------------------------------------------------------------
-__global__ void k_set_equilibrium3d(const __grid_constant__ AuxArgs a, void *f, int inst,
-                                    const double *__restrict__ rho, const double *__restrict__ ux,
-                                    const double *__restrict__ uy, const double *__restrict__ uz)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int zy = blockIdx.y;  // z * Ly + y
-    if (x >= a.Lx) return;
-    const int Q1 = ax_q(a.tab);
-    const long long node = (long long)zy * a.Lx + x;
-    const double r = rho[node];
-    const long long base = (long long)inst * a.inst_stride + (long long)zy * a.pitch + x;
-    const bool f64 = a.prec == GLBM_FP64;
-    // per node: E^x (FP64 storage) or E^x - W^x (FP32 deviations), and E^y - W^y
-    double exs[GLBM_MAXQA], dys[GLBM_MAXQA], dzs[GLBM_MAXQA];
-    eq_dev_all_rt(a.tab, ux[node], exs);
-    eq_dev_all_rt(a.tab, uy[node], dys);
-    eq_dev_all_rt(a.tab, uz[node], dzs);
-    if (f64)
-        for (int i = 0; i < Q1; ++i) exs[i] += a.tab.W[i];
-    for (int iz = 0; iz < Q1; ++iz) {
-        const double wz = a.tab.W[iz], dz = dzs[iz];
-        for (int iy = 0; iy < Q1; ++iy) {
-            const double wy = a.tab.W[iy], dy = dys[iy];
-            // per row: A = rho E^y E^z and B = rho E^y E^z - W^y W^z =
-            // (rho - 1) W^y W^z + rho (d^y E^z + W^y d^z) (no cancellation);
-            // then rho E^x E^y E^z = E^x A, and in deviations W^x B + d^x A
-            const double A = r * ((wy + dy) * (wz + dz));
-            const double B = fma(r - 1.0, wy * wz, r * fma(dy, wz + dz, wy * dz));
-            const long long row = base + (long long)((iz * Q1 + iy) * Q1) * a.plane;
-            if (f64) {
-                double *out = static_cast<double *>(f) + row;
-                for (int ix = 0; ix < Q1; ++ix) out[(long long)ix * a.plane] = exs[ix] * A;
-            } else {
-                float *out = static_cast<float *>(f) + row;
-                for (int ix = 0; ix < Q1; ++ix)
-                    out[(long long)ix * a.plane] = (float)fma(exs[ix], A, a.tab.W[ix] * B);
-            }
-        }
-    }
-}
-
 }  // namespace
-
-cudaError_t glbm_launch_set_equilibrium3d(const AuxArgs &a, void *f, int inst, const double *rho,
-                                          const double *ux, const double *uy, const double *uz,
-                                          cudaStream_t s)
-{
-    dim3 grid((a.Lx + 127) / 128, a.Ly * a.Lz);
-    k_set_equilibrium3d<<<grid, 128, 0, s>>>(a, f, inst, rho, ux, uy, uz);
-    return cudaGetLastError();
-}
-
-cudaError_t glbm_launch_set_equilibrium(const AuxArgs &a, void *f, int inst, const double *rho,
-                                        const double *ux, const double *uy, cudaStream_t s)
-{
-    dim3 grid((a.Lx + 127) / 128, a.Ly);
-    k_set_equilibrium<<<grid, 128, 0, s>>>(a, f, inst, rho, ux, uy);
-    return cudaGetLastError();
-}
 
 cudaError_t glbm_launch_set_populations(const AuxArgs &a, void *f, int inst, const double *src,
                                         cudaStream_t s)

@@ -304,8 +304,11 @@ struct AuxArgs {
     long long plane, inst_stride;
     int Lz;               // nodes along z (3D; 1 otherwise)
 };
-cudaError_t glbm_launch_set_equilibrium(const AuxArgs &a, void *f, int inst, const double *rho,
-                                        const double *ux, const double *uy, cudaStream_t s);
+// Equilibrium of the fields rho (null: 1) and u_x, u_y, u_z (null: 0) of one
+// instance (glbm_equilibrium.cu; f: its populations).
+cudaError_t glbm_launch_set_equilibrium(const AuxArgs &a, void *f, const double *rho,
+                                        const double *ux, const double *uy, const double *uz,
+                                        cudaStream_t s);
 cudaError_t glbm_launch_set_populations(const AuxArgs &a, void *f, int inst, const double *src,
                                         cudaStream_t s);
 cudaError_t glbm_launch_get_populations(const AuxArgs &a, const void *f, int inst, double *dst,
@@ -321,10 +324,6 @@ cudaError_t glbm_launch_moments(const AuxArgs &a, const void *f, double *rw, con
                                 cudaStream_t s);
 cudaError_t glbm_launch_moments1d(const AuxArgs &a, const void *f, const MomPtrs &out,
                                   cudaStream_t s);
-// 3D: initial equilibrium with u_z.
-cudaError_t glbm_launch_set_equilibrium3d(const AuxArgs &a, void *f, int inst, const double *rho,
-                                          const double *ux, const double *uy, const double *uz,
-                                          cudaStream_t s);
 // Channel diagnostics (Sec. 5.3, 5.4) of one instance from its moment fields
 // (mom: rho, then u_x): prof[0..Ly) the row
 // means of u_x, prof[Ly..2Ly) of rho u_x, stats[GLBM_CH_*] the scalars.
