@@ -1174,6 +1174,32 @@ static glbm_status step_1d_instance(glbm_ctx *c, int i, int64_t n, int64_t *comp
     return GLBM_OK;
 }
 
+// n steps of every 1D instance in one launch of clusters, from the current buffer
+// into the other one. *done is false, and the state unchanged, where the cluster
+// does not hold the lattice or a node left the positivity domain: the instances
+// are then stepped one after another (step_1d_instance), which stops at the
+// failing step.
+static glbm_status step_1d_clusters(glbm_ctx *c, int64_t n, bool *done)
+{
+    *done = false;
+    AuxArgs a = aux_args(c, 0);
+    a.inst_stride = c->n_inst > 1 ? c->geo[1].off : 0;
+    int ok = 0;
+    CUDA_TRY(glbm_launch_run1d_cluster(a, inst_ptr(c, c->cur, 0), inst_ptr(c, 1 - c->cur, 0), c->n_inst,
+                                       n, c->d_status, c->stream, &ok));
+    if (!ok) return GLBM_OK;
+    c->launches += 1;
+    glbm_status st = read_status(c);
+    if (st != GLBM_OK) return st;
+    if (c->h_status[ST_FLAGS] & ST_UNSTABLE) {
+        CUDA_TRY(clear_unstable(c));
+        return GLBM_OK;
+    }
+    c->cur = 1 - c->cur;
+    *done = true;
+    return GLBM_OK;
+}
+
 // Enqueue n (< 2^31) 2D or 3D steps of every instance; returns the steps
 // completed (each step's last launch counts itself, and once a step has left
 // the positivity domain the launches of later steps do nothing).
@@ -1247,9 +1273,14 @@ extern "C" glbm_status glbm_step(glbm_ctx *c, int64_t n)
     int64_t done = 0;  // steps of every instance completed by this call
     bool bad = false;
     if (c->dims == 1) {
-        // instances one after another; each stops at its own failing step
+        bool run = false;
+        if (n > 0 && !c->halted) {
+            glbm_status st = step_1d_clusters(c, n, &run);
+            if (st != GLBM_OK) return st;
+        }
+        // else instances one after another; each stops at its own failing step
         done = n;
-        for (int i = 0; i < c->n_inst; ++i) {
+        for (int i = 0; i < c->n_inst && !run; ++i) {
             int64_t k = 0;
             glbm_status st = step_1d_instance(c, i, n, &k);
             if (st != GLBM_OK) return st;

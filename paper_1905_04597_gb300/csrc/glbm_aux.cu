@@ -5,7 +5,7 @@
 #include <algorithm>
 #include <mutex>
 
-#include "glbm_device.cuh"
+#include "glbm_node1d.cuh"
 
 namespace {
 
@@ -227,67 +227,17 @@ __global__ void k_channel_stats(const double *__restrict__ prof, int Ly, Channel
 }
 
 // ---------------------------------------------------------------------------
-// 1D step (Sec. 5.1): pull with halfway bounce-back or periodic ends, moments,
-// equilibrium, relaxation. One thread per node.
+// 1D step (glbm_node1d.cuh), one thread per node: a launch per step, or many steps
+// of a small lattice in one CTA. Most calls take the cluster of glbm_run1d.cu; these
+// serve the lattices it does not hold and the calls whose run fails inside it.
 // ---------------------------------------------------------------------------
-template <int N, typename T>
-__device__ __forceinline__ void node1d(const AuxArgs &a, const InstParams &ip, const T *fin,
-                                       T *fout, int x, int L, long long plane, unsigned *status)
-{
-    constexpr int Q1 = 2 * N + 1;
-    constexpr bool DEV = sizeof(T) == 4;
-    using Acc = TabAcc<T>;
-    T f[Q1];
-#pragma unroll
-    for (int ix = 0; ix < Q1; ++ix) {
-        const int n = ix - N;
-        int xs = x - n, q = ix;
-        if (a.bc == GLBM_BC_PERIODIC) {
-            xs = wrap_index(xs, L);
-        } else if (xs < 0) {
-            xs = -1 - xs;
-            q = 2 * N - ix;
-        } else if (xs >= L) {
-            xs = 2 * L - 1 - xs;
-            q = 2 * N - ix;
-        }
-        f[ix] = fin[(long long)q * plane + xs];
-    }
-    T s = T(0), c = T(0), sj = T(0), cj = T(0);
-#pragma unroll
-    for (int ix = 0; ix < Q1; ++ix) acc2(s, c, f[ix]);
-#pragma unroll
-    for (int n = 1; n <= N; ++n) acc2(sj, cj, T(n) * (f[N + n] - f[N - n]));
-    const T m0 = s + c;
-    const T rho = DEV ? T(1) + m0 : m0;
-    const T drho = DEV ? m0 : m0 - T(1);
-    const T j = sj + cj;
-    T u = j / rho;
-    // FP32: u = j / (1 + delta rho) from the unrounded density, by one
-    // correction with the residual (j - u) - u delta rho (j - u is exact)
-    if (DEV) u += fma(-u, drho, j - u) / rho;
-    const T umax = (T)(0.816496580927726 * N);
-    if (!(rho > T(0)) || !(fabs(u) <= umax)) flag_unstable(status);
-    T d[Q1];
-    eq_dev_all<N, T>(a.tab, u, d);
-    const T om = DEV ? (T)ip.omega_f : (T)ip.omega;
-#pragma unroll
-    for (int ix = 0; ix < Q1; ++ix) {
-        const T w = Acc::W(a.tab, ix);
-        // FP32: delta f^eq = d + drho (W + d), the momentum-carrying d unscaled
-        // by a rounded rho; FP64: f^eq = rho (W + d)
-        const T eq = DEV ? fma(drho, w + d[ix], d[ix]) : rho * (w + d[ix]);
-        fout[(long long)ix * plane + x] = fma(om, eq - f[ix], f[ix]);  // f + omega (f^eq - f)
-    }
-}
-
 template <int N, typename T>
 __global__ void k_step1d(const __grid_constant__ AuxArgs a, const T *__restrict__ fin,
                          T *__restrict__ fout, int inst, unsigned *status)
 {
     if (step_halted(status)) return;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x < a.Lx) node1d<N, T>(a, a.ip[inst], fin, fout, x, a.Lx, a.plane, status);
+    if (x < a.Lx) node1d_at<N, T>(a, a.ip[inst], fin, fout, x, a.Lx, a.plane, status);
     finish_step(status);
 }
 
@@ -314,7 +264,7 @@ __global__ void k_run1d_resident(const __grid_constant__ AuxArgs a, T *__restric
     long long done = 0;
     while (done < steps) {
         for (int x = threadIdx.x; x < L; x += blockDim.x)
-            node1d<N, T>(a, a.ip[inst], A, B, x, L, L, status);
+            node1d_at<N, T>(a, a.ip[inst], A, B, x, L, L, status);
         __syncthreads();  // the step's flags (global atomics of this block) are visible
         T *tmp = A;
         A = B;
@@ -362,7 +312,11 @@ cudaError_t launch_resident_n(const AuxArgs &a, T *f, int inst, long long steps,
     cudaError_t e = cudaFuncSetAttribute(k_run1d_resident<N, T>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int threads = a.Lx >= 1024 ? 1024 : ((a.Lx + 31) / 32) * 32;
+    cudaFuncAttributes fa;  // FP64 of the higher levels: fewer threads than 1024 fit
+    e = cudaFuncGetAttributes(&fa, k_run1d_resident<N, T>);
+    if (e != cudaSuccess) return e;
+    const int most = fa.maxThreadsPerBlock / 32 * 32;
+    const int threads = std::min(most, ((a.Lx + 31) / 32) * 32);
     k_run1d_resident<N, T><<<1, threads, smem, s>>>(a, f, inst, steps, status);
     return cudaGetLastError();
 }

@@ -340,6 +340,11 @@ cudaError_t glbm_launch_field_sums(const double *fields, int nfields, long long 
 int glbm_field_sum_blocks(long long n);
 cudaError_t glbm_launch_step1d(const AuxArgs &a, const void *fin, void *fout, int inst,
                                unsigned *status, cudaStream_t s);
+// `steps` steps of n_inst 1D lattices (instances a.inst_stride elements apart) from f
+// into out, each on a cluster of CTAs (glbm_run1d.cu). *ok is 0, and nothing was
+// launched, for lattices the cluster does not hold.
+cudaError_t glbm_launch_run1d_cluster(const AuxArgs &a, const void *f, void *out, int n_inst,
+                                      long long steps, unsigned *status, cudaStream_t s, int *ok);
 cudaError_t glbm_launch_run1d_resident(const AuxArgs &a, void *f, int inst, long long steps,
                                        unsigned *status, cudaStream_t s, int *ok);
 
