@@ -817,8 +817,7 @@ extern "C" glbm_status glbm_set_populations(glbm_ctx *c, int inst, const double 
         CUDA_TRY(cudaMemcpyAsync(c->d_stage, f, n * 8, cudaMemcpyHostToDevice, c->stream));
         src = c->d_stage;
     }
-    CUDA_TRY(glbm_launch_set_populations(aux_args(c, inst), inst_ptr(c, c->cur, inst), 0, src,
-                                         c->stream));
+    CUDA_TRY(glbm_launch_set_populations(aux_args(c, inst), inst_ptr(c, c->cur, inst), src, c->stream));
     c->launches += 1;
     CUDA_TRY(set_clock(c, 0));
     CUDA_TRY(clear_unstable(c));
@@ -838,8 +837,7 @@ extern "C" glbm_status glbm_get_populations(glbm_ctx *c, int inst, double *f, in
         if (st != GLBM_OK) return st;
         dst = c->d_stage;
     }
-    CUDA_TRY(glbm_launch_get_populations(aux_args(c, inst), inst_ptr(c, c->cur, inst), 0, dst,
-                                         c->stream));
+    CUDA_TRY(glbm_launch_get_populations(aux_args(c, inst), inst_ptr(c, c->cur, inst), dst, c->stream));
     c->launches += 1;
     if (!on_device) {
         CUDA_TRY(cudaMemcpyAsync(f, dst, n * 8, cudaMemcpyDeviceToHost, c->stream));

@@ -440,6 +440,17 @@ __device__ __forceinline__ double f2d(float x)
     return e ? __hiloint2double((int)hi, (int)(b << 29)) : 0.0;
 }
 
+// (float)x (to nearest even) by integer instructions where the result is a normal
+// float, for the same reason.
+__device__ __forceinline__ float d2f(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned e = (hi >> 20) & 0x7FFu;
+    if (e - 897u > 253u) return (float)x;  // 0, subnormal or infinite as a float, NaN
+    const unsigned b = (((hi & 0x7FFFFFFFu) - (896u << 20)) << 3) | (lo >> 29);
+    const unsigned r = b + (((lo & 0x1FFFFFFFu) + (b & 1u) + 0x0FFFFFFFu) >> 29);
+    return __uint_as_float(r | (hi & 0x80000000u));
+}
 __device__ __forceinline__ double to_f64(float x) { return f2d(x); }
 __device__ __forceinline__ double to_f64(double x) { return x; }
 

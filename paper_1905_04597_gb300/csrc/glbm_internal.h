@@ -309,9 +309,9 @@ struct AuxArgs {
 cudaError_t glbm_launch_set_equilibrium(const AuxArgs &a, void *f, const double *rho,
                                         const double *ux, const double *uy, const double *uz,
                                         cudaStream_t s);
-cudaError_t glbm_launch_set_populations(const AuxArgs &a, void *f, int inst, const double *src,
+cudaError_t glbm_launch_set_populations(const AuxArgs &a, void *f, const double *src,
                                         cudaStream_t s);
-cudaError_t glbm_launch_get_populations(const AuxArgs &a, const void *f, int inst, double *dst,
+cudaError_t glbm_launch_get_populations(const AuxArgs &a, const void *f, double *dst,
                                         cudaStream_t s);
 // Destinations of the moment fields, by the bit of GLBM_M_*; null: not wanted.
 struct MomPtrs {
