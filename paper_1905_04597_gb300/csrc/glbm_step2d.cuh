@@ -45,7 +45,8 @@ struct Step2D {
     using A = TabAcc<T>;
 
     struct Smem {
-        T part[R][G][6][32];  // (s, c) pairs of delta rho, j_x, j_y per row and group
+        T part[R][G][DEV ? 6 : 3][32];  // (s, c) pairs (FP64: s) of delta rho, j_x, j_y
+                                        // per row and group
         T rw[2][32];          // wall density (FP64) or its deviation (FP32): lo, hi
         T dsum[NV][2][32];    // partial wall fluxes of the NV accumulators
         // E^x - W and E^y - W of the tile's nodes, shared by the warp groups
@@ -147,6 +148,17 @@ struct Step2D {
         }
     }
 
+    // FP64 row sums of f and of xi_x f from the mirror column pairs.
+    __device__ __forceinline__ static void row_sums(const T (&v)[QX], T &rs, T &jx)
+    {
+#pragma unroll
+        for (int m = AX::M0; m <= NXL; ++m) {
+            const T p = v[AX::ipos(m)] + v[AX::ineg(m)], d = v[AX::ipos(m)] - v[AX::ineg(m)];
+            rs = m == AX::M0 ? (ZX ? p : v[NXL] + p) : rs + p;
+            jx = m == AX::M0 ? d : fma(T(AX::vmag(m)), d, jx);
+        }
+    }
+
     // One tile: columns x0..x0+31, rows y0..y0+R-1 of one instance whose
     // populations start at fin / fout; tab is the y axis's table, tabx the x
     // axis's (the same table for isotropic lattices). rwg, when set, holds the
@@ -219,16 +231,24 @@ struct Step2D {
                         }
                     }
                 }
-                T rs = T(0);
+                if constexpr (DEV) {
+                    T rs = T(0);
 #pragma unroll
-                for (int ix = 0; ix < QX; ++ix) rs += f[k][ix];
-                T jx = T(0);
+                    for (int ix = 0; ix < QX; ++ix) rs += f[k][ix];
+                    T jx = T(0);
 #pragma unroll
-                for (int m = AX::M0; m <= NXL; ++m)
-                    jx = fma(T(AX::vmag(m)), f[k][AX::ipos(m)] - f[k][AX::ineg(m)], jx);
-                acc2(s_r, c_r, rs);
-                acc2(s_x, c_x, jx);
-                if (ny != 0) acc2(s_y, c_y, mul_rn(T(ny), rs));
+                    for (int m = AX::M0; m <= NXL; ++m)
+                        jx = fma(T(AX::vmag(m)), f[k][AX::ipos(m)] - f[k][AX::ineg(m)], jx);
+                    acc2(s_r, c_r, rs);
+                    acc2(s_x, c_x, jx);
+                    if (ny != 0) acc2(s_y, c_y, mul_rn(T(ny), rs));
+                } else {
+                    T rs, jx;
+                    row_sums(f[k], rs, jx);
+                    s_r = k == 0 ? rs : s_r + rs;
+                    s_x = k == 0 ? jx : s_x + jx;
+                    if (ny != 0) s_y = fma(to_f64((float)ny), rs, s_y);
+                }
             }
         }
         // ---- phase 2: moments, equilibrium, relaxation, store --------------
@@ -245,6 +265,20 @@ struct Step2D {
                 C_x = c_x;
                 C_y = c_y;
             }
+        } else if constexpr (!DEV) {
+            sm.part[r][g][0][lane] = s_r;
+            sm.part[r][g][1][lane] = s_x;
+            sm.part[r][g][2][lane] = s_y;
+            __syncthreads();
+            S_r = sm.part[r][0][0][lane];
+            S_x = sm.part[r][0][1][lane];
+            S_y = sm.part[r][0][2][lane];
+#pragma unroll
+            for (int gi = 1; gi < G; ++gi) {
+                S_r += sm.part[r][gi][0][lane];
+                S_x += sm.part[r][gi][1][lane];
+                S_y += sm.part[r][gi][2][lane];
+            }
         } else {
             sm.part[r][g][0][lane] = s_r;
             sm.part[r][g][1][lane] = c_r;
@@ -258,19 +292,17 @@ struct Step2D {
                 acc2(S_r, C_r, sm.part[r][gi][0][lane]);
                 acc2(S_x, C_x, sm.part[r][gi][2][lane]);
                 acc2(S_y, C_y, sm.part[r][gi][4][lane]);
-                if (DEV) {
-                    C_r += sm.part[r][gi][1][lane];
-                    C_x += sm.part[r][gi][3][lane];
-                    C_y += sm.part[r][gi][5][lane];
-                }
+                C_r += sm.part[r][gi][1][lane];
+                C_x += sm.part[r][gi][3][lane];
+                C_y += sm.part[r][gi][5][lane];
             }
         }
-        const T m0 = S_r + C_r;            // FP32: delta rho; FP64: rho
+        const T m0 = DEV ? S_r + C_r : S_r;  // FP32: delta rho; FP64: rho
         const T rho = DEV ? T(1) + m0 : m0;
         const T drho = DEV ? m0 : m0 - T(1);
         const T inv_rho = T(1) / rho;
-        T jx = S_x + C_x;
-        const T jy = S_y + C_y;
+        T jx = DEV ? S_x + C_x : S_x;
+        const T jy = DEV ? S_y + C_y : S_y;
         // Guo's form: the equilibrium takes u = (j + g/2) / rho
         const T gh = GUO ? (DEV ? (T)ip.g_half_f : (T)ip.g_half) : T(0);
         if constexpr (GUO) jx += gh;
@@ -293,7 +325,7 @@ struct Step2D {
             ux = fma(fma(-ux, drho, rx) + dux, inv_rho, ux);
             uy = fma(fma(-uy, drho, (S_y - uy) + C_y) + duy, inv_rho, uy);
         }
-        if (active) {
+        if (active && (DEV || g == 0)) {
             // sqrt(2/3) N per axis: positivity bound (Sec. 3), twice that in
             // the half-spacing units of a 2N+2 axis
             const T umax = (T)(0.816496580927726 * (ZY ? 2 * N : N));
@@ -431,42 +463,49 @@ struct Step2D {
                         op[(ix + 1) * plane] = hi2(v2);
                     }
                 }
+                if constexpr (!DEV) {
+                    // f^eq - f0 in one fused rounding, then the force term (skipped
+                    // without a force), then f0 + omega (f^eq + F/omega - f0): three
+                    // FP64 instructions, two without a force
+                    T d[QX];
 #pragma unroll
-                for (int ix = (DEV ? QX - (QX & 1) : 0); ix < QX; ++ix) {
+                    for (int ix = 0; ix < QX; ++ix) d[ix] = fma(ex[ix], rey, -f[k][ix]);
+                    if (GUO || gto != T(0)) {
+#pragma unroll
+                        for (int ix = 0; ix < QX; ++ix) {
+                            const int nx = AX::vel(ix);
+                            if constexpr (GUO)
+                                d[ix] = fma(A::W(tabx, ix), fma(T(nx), grA, T(AX::ck(ix)) * grB), d[ix]);
+                            else if (nx != 0)
+                                d[ix] = fma(A::WN(tabx, ix), gr, d[ix]);
+                        }
+                    }
+#pragma unroll
+                    for (int ix = 0; ix < QX; ++ix) op[ix * plane] = fma(om, d[ix], f[k][ix]);
+                }
+#pragma unroll
+                for (int ix = (DEV ? QX - (QX & 1) : QX); ix < QX; ++ix) {
                     const int nx = AX::vel(ix);
                     const T f0 = f[k][ix];
-                    T v;
-                    if (DEV) {
-                        const T Bn = GUO ? fma(T(nx), grA, fma(T(AX::ck(ix)), grB, B))
-                                         : (nx != 0 ? fma(T(nx), gr, B) : B);
-                        // split FP32 tiles read E^x - W where it is used (fewer registers)
-                        const T dxv = DX_SHARED ? sm.eqx[r][ix][lane] : dx[ix];
-                        // delta f^eq = d^x W^y + E^x B + F/omega: the momentum-
-                        // carrying d^x meets only the float weight W^y (whose row
-                        // sum is exactly 1); a rounded rho e^y there would scale
-                        // the momentum by a fixed 1 + O(2^-24) at every step of a
-                        // steady flow. f^eq is never rounded at the scale of f:
-                        // r = f0 - d^x W^y cancels (one fused rounding, of a small
-                        // value when the flow runs along x), t1 holds the rest of
-                        // f^eq plus the dither (half an ulp of f0, over omega),
-                        // and the store f0 + omega (t1 - r) is one rounding that
-                        // sees the whole dither: zero-mean.
-                        const float u = dither_pick(ix, ua, ub, -ua, -ub);
-                        const T dith = (T)dither_ulp((float)f0, u);
-                        const T t1 = fma(dxv, B, fma(A::W(tabx, ix), Bn, dith));
-                        const T r = fma(dxv, nwy, f0);
-                        v = fma(om, t1 - r, f0);
-                    } else {
-                        // f^eq - f0 in one fused rounding, then the force term,
-                        // then f0 + omega (f^eq + F/omega - f0): three FP64
-                        // instructions (two without a force term)
-                        T d = fma(ex[ix], rey, -f0);
-                        if constexpr (GUO)
-                            d = fma(A::W(tabx, ix), fma(T(nx), grA, T(AX::ck(ix)) * grB), d);
-                        else if (nx != 0)
-                            d = fma(A::WN(tabx, ix), gr, d);
-                        v = fma(om, d, f0);
-                    }
+                    const T Bn = GUO ? fma(T(nx), grA, fma(T(AX::ck(ix)), grB, B))
+                                     : (nx != 0 ? fma(T(nx), gr, B) : B);
+                    // split FP32 tiles read E^x - W where it is used (fewer registers)
+                    const T dxv = DX_SHARED ? sm.eqx[r][ix][lane] : dx[ix];
+                    // delta f^eq = d^x W^y + E^x B + F/omega: the momentum-
+                    // carrying d^x meets only the float weight W^y (whose row
+                    // sum is exactly 1); a rounded rho e^y there would scale
+                    // the momentum by a fixed 1 + O(2^-24) at every step of a
+                    // steady flow. f^eq is never rounded at the scale of f:
+                    // r = f0 - d^x W^y cancels (one fused rounding, of a small
+                    // value when the flow runs along x), t1 holds the rest of
+                    // f^eq plus the dither (half an ulp of f0, over omega),
+                    // and the store f0 + omega (t1 - r) is one rounding that
+                    // sees the whole dither: zero-mean.
+                    const float u = dither_pick(ix, ua, ub, -ua, -ub);
+                    const T dith = (T)dither_ulp((float)f0, u);
+                    const T t1 = fma(dxv, B, fma(A::W(tabx, ix), Bn, dith));
+                    const T r = fma(dxv, nwy, f0);
+                    const T v = fma(om, t1 - r, f0);
                     op[ix * plane] = v;
                 }
             }

@@ -131,32 +131,32 @@ __global__ void __launch_bounds__((SMALL_NB * AxisVel<N, ZY>::Q + 31) / 32 * 32)
     }
     // moments: row sums, then the sums over the rows in the order of G0 warp groups
     if (row) {
-        double r = 0.0, jx = 0.0;
-#pragma unroll
-        for (int ix = 0; ix < QX; ++ix) r += f[ix];
-#pragma unroll
-        for (int m = AX::M0; m <= NXL; ++m)
-            jx = fma((double)AX::vmag(m), f[AX::ipos(m)] - f[AX::ineg(m)], jx);
+        double r, jx;
+        S::row_sums(f, r, jx);
         rs[i][j] = r;
         jr[i][j] = jx;
     }
     __syncthreads();
     for (int t = i; t < 3 * G0; t += Q1) {
         const int k = t / G0, g = t - k * G0;
-        double s = 0.0;
         if (row) {
+            double s = k == 0 ? rs[g][j] : k == 1 ? jr[g][j] : (double)AY::vel(g) * rs[g][j];
 #pragma unroll 4
-            for (int q = g; q < Q1; q += G0)
-                s += k == 0 ? rs[q][j] : k == 1 ? jr[q][j] : mul_rn((double)AY::vel(q), rs[q][j]);
+            for (int q = g + G0; q < Q1; q += G0) {
+                if (k < 2)
+                    s += k == 0 ? rs[q][j] : jr[q][j];
+                else if (AY::vel(q) != 0)
+                    s = fma(to_f64((float)AY::vel(q)), rs[q][j], s);
+            }
             (G0 == 1 ? tot[k][j] : part[t][j]) = s;
         }
     }
     __syncthreads();
     if constexpr (G0 > 1) {
         if (i < 3) {
-            double s = 0.0;
+            double s = part[i * G0][j];
 #pragma unroll
-            for (int g = 0; g < G0; ++g) s += part[i * G0 + g][j];
+            for (int g = 1; g < G0; ++g) s += part[i * G0 + g][j];
             tot[i][j] = s;
         }
         __syncthreads();
