@@ -447,7 +447,8 @@ glbm_status glbm_autotune(glbm_ctx *ctx, int reps, double *us);
  * per column and wall into a small device buffer (mode 1, one more launch per
  * step). The sums are the same, in the same order: both modes give identical
  * results. A new context takes mode 1 where the tiles near the walls would
- * repeat the sums for more than a tenth of a step's own loads (high levels,
+ * repeat the sums for more than a tenth of a step's own loads (in FP32 up to k = 7,
+ * whose steps then take dataflow chunks, more than a fifth: high levels,
  * narrow channels), else mode 0. glbm_set_wall_launch sets the mode (0 or 1;
  * -1 restores that default; GLBM_E_INVAL otherwise, GLBM_E_UNSUPPORTED for a
  * context without walls, a batch of mixed levels or a 3D context;

@@ -458,8 +458,12 @@ static glbm_status ensure_stage(glbm_ctx *c, size_t n)
 // Whether the wall densities of a step get a launch of their own (k_wall_rho,
 // once per column and wall) instead of the prologue of every tile within reach
 // of a wall: when those tiles, at one node row each, would repeat the wall sums
-// for more than a tenth of the step's own loads. Uniform 2D lattices with walls.
-static bool wall_rho_pays(int N, int NX, int zv, int Ly)
+// for more than 1/share of the step's own loads. Uniform 2D lattices with walls.
+// The share is a tenth, and a fifth in FP32 up to level 8, where a step without
+// that launch takes dataflow chunks (GB300, us per step, own launch against tiles
+// with dataflow: D1Q3 x D1Q8 1000 x 200 x 3 at 14 % 26.6 and 22.2, D2Q121 256 x 128
+// at 11 % 10.1 and 9.2, D2Q289 1024 x 128 x 8 at 26 % 476 and 591).
+static bool wall_rho_pays(int N, int NX, int zv, int Ly, int share)
 {
     const bool zy = (zv & GLBM_ZV_Y) != 0, zx = (zv & GLBM_ZV_X) != 0;
     // largest y speed and number of (velocity, row) pairs of one wall: the 2N+1
@@ -468,7 +472,7 @@ static bool wall_rho_pays(int N, int NX, int zv, int Ly)
     const long long npair = zy ? (long long)(N + 1) * (N + 1) : (long long)N * (N + 1) / 2;
     const long long qx = zx ? 2 * NX + 2 : 2 * NX + 1, qy = zy ? 2 * N + 2 : 2 * N + 1;
     const long long repeated = 2 * std::min<long long>(vmax, Ly) * npair * qx;
-    return 10 * repeated > (long long)Ly * qx * qy;
+    return share * repeated > (long long)Ly * qx * qy;
 }
 
 static bool wall_rho_possible(const glbm_ctx *c)
@@ -478,7 +482,8 @@ static bool wall_rho_possible(const glbm_ctx *c)
 static bool wall_rho_launch(const glbm_ctx *c)
 {
     const Geo &g = c->geo[0];
-    return wall_rho_possible(c) && wall_rho_pays(g.N, g.NX, g.zv, g.Ly);
+    const int share = c->prec == GLBM_FP32_DEV && g.N <= GLBM_MAXN_2N1 ? 5 : 10;
+    return wall_rho_possible(c) && wall_rho_pays(g.N, g.NX, g.zv, g.Ly, share);
 }
 static glbm_status alloc_wall_rho(glbm_ctx *c)
 {
@@ -710,6 +715,11 @@ extern "C" glbm_status glbm_batch_create(const glbm_config *cfgs, int n, void *s
     glbm_ctx *c = new (std::nothrow) glbm_ctx();
     if (!c) return fail(GLBM_E_NOMEM, "host allocation failed");
     c->hetero = true;
+    // batches hold narrow channels: the entry of the default's G (same results) that
+    // was faster there (GB300, 64 channels of 64 columns, us per launch): (4, 1, 2)
+    // 76.4 against (4, 2, 1) 83.8 at N = 6, (5, 1, 1) 46.3 against (5, 1, 2) 49.4 at 7
+    c->tile[6] = 2;
+    c->tile[7] = 1;
     glbm_status st = finish_create(c, cfgs, n, stream);
     if (st == GLBM_OK) st = build_items(c);
     if (st != GLBM_OK) {
