@@ -10,12 +10,13 @@
 // What bounds it: FP64 needs two instructions and a conversion per population on a
 // pipe that issues two per cycle and SM, fourteen times the time of the stores. FP32
 // deviations are formed in float pairs (value = h + l, 48 bits) on the FP32 pipe
-// instead: the result is rounded to float once from a value exact to 2^-46 of its
-// terms, which differs from the rounding of the FP64 value about once in 2^20
-// populations, at a tie. Fields outside 1e-18..1e18 in magnitude (or not finite)
-// take FP64 per node. Measured on GB300, FP32: D2Q81 512 x 256 95 -> 26 us, D2Q289
-// 1024 x 128 311 -> 75 us, D3Q125 250 x 61 x 45 815 -> 227 us, D1Q3 x D1Q28 200 nodes
-// (FP64) 25 -> 10 us; large FP64 lattices stay on the FP64 pipe (D2Q81 54 us).
+// instead: the value before the rounding to float is exact to 2^-43 of its terms, and
+// where the rounding could go either way within 2^-41 (about one population in 2^16)
+// it is formed in FP64, so every stored float is that of the FP64 formula. Fields
+// outside 1e-18..1e18 in magnitude (or not finite) take FP64. Measured on GB300, FP32:
+// D2Q81 512 x 256 95 -> 29 us, D2Q289 1024 x 128 311 -> 80 us, D3Q125 250 x 61 x 45
+// 815 -> 256 us, D1Q3 x D1Q28 200 nodes (FP64) 25 -> 10 us; large FP64 lattices stay
+// on the FP64 pipe (D2Q81 54 us).
 #include "glbm_device.cuh"
 
 namespace {
@@ -75,15 +76,19 @@ struct F32 {
 
 // Table of one axis in the arithmetic's values: rest weights by velocity index, and
 // the even and odd coefficients of every mirror pair (Ce[m][i], i = 0..N-1 for v^(i+1)).
-template <class V>
+// M: the highest level it holds (kernel parameters of 5 KB at 8, 12 KB at 13).
+template <class V, int M>
 struct EqAxis {
     int N, zv;
-    V W[GLBM_MAXQA];
-    V Ce[GLBM_MAXN + 1][GLBM_MAXN], Co[GLBM_MAXN + 1][GLBM_MAXN];
+    V W[2 * M + 2];
+    V Ce[M + 1][M], Co[M + 1][M];
 };
-template <class V>
+struct NoAxis {};
+template <class V, int M>
 struct EqArgs {
-    EqAxis<V> y, x;  // 3D: y holds for z too
+    EqAxis<V, M> y, x;  // 3D: y holds for z too
+    // float pairs: the FP64 tables too
+    std::conditional_t<std::is_same<V, df>::value, EqAxis<double, M>, NoAxis> y64, x64;
     const double *rho, *u[3];  // null: 1, 0
     void *f;
     int Lx, nodes, pitch, dims;
@@ -91,8 +96,8 @@ struct EqArgs {
 };
 
 // E - W of the mirror pair m of one axis (plus: the positive velocity).
-template <class P>
-__device__ __forceinline__ void eq_pair(const EqAxis<typename P::V> &t, int m, typename P::V u,
+template <class P, int M>
+__device__ __forceinline__ void eq_pair(const EqAxis<typename P::V, M> &t, int m, typename P::V u,
                                         typename P::V &plus, typename P::V &minus)
 {
     using V = typename P::V;
@@ -112,63 +117,62 @@ __device__ __forceinline__ void eq_pair(const EqAxis<typename P::V> &t, int m, t
     minus = P::fma_(P::neg(u), o, e);
 }
 
-// W^x B + d^x A rounded once to float.
-__device__ __forceinline__ float eq_dev(df w, df B, df d, df A)
+// Population (iz, iy, ix) of node n in FP64.
+template <int M>
+__device__ __noinline__ float eq_exact(const EqArgs<df, M> &a, int n, int iz, int iy, int ix)
+{
+    const auto dev = [](const EqAxis<double, M> &t, double u, int i) {
+        const int vel = t.zv ? 2 * i - (2 * t.N + 1) : i - t.N, av = vel < 0 ? -vel : vel;
+        const int m = t.zv ? (av - 1) / 2 : av;
+        const double v = u * u;
+        double e = t.Ce[m][t.N - 1], o = t.Co[m][t.N - 1];
+        for (int k = t.N - 2; k >= 0; --k) {
+            e = fma(e, v, t.Ce[m][k]);
+            o = fma(o, v, t.Co[m][k]);
+        }
+        e = mul_rn(e, v);
+        return vel == 0 ? e : fma(vel > 0 ? u : -u, o, e);
+    };
+    const double r = a.rho ? a.rho[n] : 1.0;
+    double A = r, B = r - 1.0;
+    if (a.dims >= 2) {
+        const double wy = a.y64.W[iy], dy = dev(a.y64, a.u[1] ? a.u[1][n] : 0.0, iy);
+        if (a.dims == 2) {
+            A = r * (wy + dy);
+            B = fma(r - 1.0, wy, mul_rn(r, dy));
+        } else {
+            const double wz = a.y64.W[iz], dz = dev(a.y64, a.u[2] ? a.u[2][n] : 0.0, iz);
+            A = r * mul_rn(wy + dy, wz + dz);
+            B = fma(r - 1.0, mul_rn(wy, wz), mul_rn(r, fma(dy, wz + dz, mul_rn(wy, dz))));
+        }
+    }
+    return (float)fma(dev(a.x64, a.u[0] ? a.u[0][n] : 0.0, ix), A, mul_rn(a.x64.W[ix], B));
+}
+
+// W^x B + d^x A rounded once to float; false where the rounding is too close to call.
+__device__ __forceinline__ bool eq_dev(df w, df B, df d, df A, float &out)
 {
     const float p = __fmul_rn(w.h, B.h), q = __fmul_rn(d.h, A.h);
     const float pe = fmaf(w.l, B.h, fmaf(w.h, B.l, fmaf(w.h, B.h, -p)));
     const float qe = fmaf(d.l, A.h, fmaf(d.h, A.l, fmaf(d.h, A.h, -q)));
     const float s = p + q, t = s - p;
-    const float e = (p - (s - t)) + (q - t);
-    return s + (e + (pe + qe));
+    const float e = ((p - (s - t)) + (q - t)) + (pe + qe);
+    const float tol = 0x1p-41f * (fabsf(p) + fabsf(q));
+    out = s + (e - tol);
+    return out == s + (e + tol);
 }
 
 constexpr int EQ_WARPS = 4;
 
-// One node of FP32 storage entirely in FP64 (out-of-range fields).
-__device__ __noinline__ void eq_node_f64(const EqArgs<df> &a, int n, long long base)
-{
-    const int Qx = 2 * a.x.N + 1 + a.x.zv, Qy = a.dims >= 2 ? 2 * a.y.N + 1 + a.y.zv : 1;
-    const int Qz = a.dims == 3 ? Qy : 1;
-    const auto val = [](df t) { return (double)t.h + (double)t.l; };
-    const auto dev = [&](const EqAxis<df> &t, double u, int i) {
-        const int vel = t.zv ? 2 * i - (2 * t.N + 1) : i - t.N, av = vel < 0 ? -vel : vel;
-        const int m = t.zv ? (av - 1) / 2 : av;
-        const double v = u * u;
-        double e = 0.0, o = 0.0;
-        for (int k = t.N - 1; k >= 0; --k) {
-            e = fma(e, v, val(t.Ce[m][k]));
-            o = fma(o, v, val(t.Co[m][k]));
-        }
-        e *= v;
-        return vel == 0 ? e : fma(vel > 0 ? u : -u, o, e);
-    };
-    const double r = a.rho ? a.rho[n] : 1.0, ux = a.u[0] ? a.u[0][n] : 0.0;
-    const double uy = a.u[1] ? a.u[1][n] : 0.0, uz = a.u[2] ? a.u[2][n] : 0.0;
-    float *const out = static_cast<float *>(a.f) + base;
-    for (int iz = 0; iz < Qz; ++iz) {
-        const double wz = a.dims == 3 ? val(a.y.W[iz]) : 1.0;
-        const double dz = a.dims == 3 ? dev(a.y, uz, iz) : 0.0;
-        for (int iy = 0; iy < Qy; ++iy) {
-            const double wy = a.dims >= 2 ? val(a.y.W[iy]) : 1.0;
-            const double dy = a.dims >= 2 ? dev(a.y, uy, iy) : 0.0;
-            const double A = r * ((wy + dy) * (wz + dz));
-            const double B = fma(r - 1.0, wy * wz, r * fma(dy, wz + dz, wy * dz));
-            for (int ix = 0; ix < Qx; ++ix)
-                out[(long long)((iz * Qy + iy) * Qx + ix) * a.plane] =
-                    (float)fma(dev(a.x, ux, ix), A, val(a.x.W[ix]) * B);
-        }
-    }
-}
-
-template <class P>
-__global__ void __launch_bounds__(32 * EQ_WARPS) k_equilibrium(const __grid_constant__ EqArgs<typename P::V> a)
+template <class P, int M>
+__global__ void __launch_bounds__(32 * EQ_WARPS)
+    k_equilibrium(const __grid_constant__ EqArgs<typename P::V, M> a)
 {
     using V = typename P::V;
     constexpr bool F = std::is_same<V, df>::value;  // float pairs
     __shared__ V in[5][32];                  // u_x, u_y, u_z, rho, rho - 1
-    __shared__ V dx[GLBM_MAXQA][32];         // FP32: E^x - W^x; FP64: E^x
-    __shared__ V dy[GLBM_MAXQA][32], dz[2 * GLBM_MAXN_3D + 1][32];
+    __shared__ V dx[2 * GLBM_MAXN_2N1 + 2][32];  // FP32: E^x - W^x; FP64: E^x
+    __shared__ V dy[2 * M + 2][32], dz[2 * GLBM_MAXN_3D + 1][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int n = blockIdx.x * 32 + lane, nc = n < a.nodes ? n : a.nodes - 1;
     const int row = nc / a.Lx, x = nc - row * a.Lx;
@@ -200,7 +204,7 @@ __global__ void __launch_bounds__(32 * EQ_WARPS) k_equilibrium(const __grid_cons
     for (int t = w; t < nx + ny + nz; t += EQ_WARPS) {
         const int ax = t < nx ? 0 : t < nx + ny ? 1 : 2;
         const int m = ax == 0 ? t : ax == 1 ? t - nx : t - nx - ny;
-        const EqAxis<V> &tab = ax == 0 ? a.x : a.y;
+        const EqAxis<V, M> &tab = ax == 0 ? a.x : a.y;
         V plus, minus;
         eq_pair<P>(tab, m, in[ax][lane], plus, minus);
         const int ip = tab.zv ? tab.N + 1 + m : tab.N + m, im = tab.N - m;
@@ -216,11 +220,11 @@ __global__ void __launch_bounds__(32 * EQ_WARPS) k_equilibrium(const __grid_cons
     const int Qx = 2 * a.x.N + 1 + a.x.zv, Qy = a.dims >= 2 ? 2 * a.y.N + 1 + a.y.zv : 1;
     const int rows = a.dims == 3 ? Qy * Qy : Qy;
     const V r = in[3][lane], r1 = in[4][lane];
-    const bool live = n < a.nodes && !((bad >> lane) & 1u);
+    const bool live = n < a.nodes, pairs = !((bad >> lane) & 1u);
     for (int j = w; j < rows; j += EQ_WARPS) {
         V A = r, B = r1;
+        const int iz = a.dims == 3 ? j / Qy : 0, iy = j - iz * Qy;
         if (a.dims >= 2) {
-            const int iz = a.dims == 3 ? j / Qy : 0, iy = j - iz * Qy;
             const V wy = a.y.W[iy], d = dy[iy][lane], E = P::add(wy, d);
             if (a.dims == 2) {
                 A = P::mul(r, E);
@@ -236,16 +240,16 @@ __global__ void __launch_bounds__(32 * EQ_WARPS) k_equilibrium(const __grid_cons
         if constexpr (F) {
             float *out = static_cast<float *>(a.f) + o;
 #pragma unroll 3
-            for (int ix = 0; ix < Qx; ++ix, out += a.plane)
-                *out = eq_dev(a.x.W[ix], B, dx[ix][lane], A);
+            for (int ix = 0; ix < Qx; ++ix, out += a.plane) {
+                float v;
+                if (!(eq_dev(a.x.W[ix], B, dx[ix][lane], A, v) && pairs)) v = eq_exact(a, nc, iz, iy, ix);
+                *out = v;
+            }
         } else {
             double *out = static_cast<double *>(a.f) + o;
 #pragma unroll 3
             for (int ix = 0; ix < Qx; ++ix, out += a.plane) *out = dx[ix][lane] * A;
         }
-    }
-    if constexpr (F) {
-        if (w == 0 && n < a.nodes && ((bad >> lane) & 1u)) eq_node_f64(a, n, base);
     }
 }
 
@@ -258,8 +262,8 @@ df host_value(double x, df *)
     return d;
 }
 
-template <class V>
-void fill_axis(const AxisTableHi &t, EqAxis<V> &e)
+template <class V, int M>
+void fill_axis(const AxisTableHi &t, EqAxis<V, M> &e)
 {
     V *const tag = nullptr;
     e.N = t.N;
@@ -272,13 +276,17 @@ void fill_axis(const AxisTableHi &t, EqAxis<V> &e)
         }
 }
 
-template <class P>
+template <class P, int M>
 cudaError_t launch_eq(const AuxArgs &a, void *f, const double *rho, const double *ux,
                       const double *uy, const double *uz, cudaStream_t s)
 {
-    EqArgs<typename P::V> e = {};
+    EqArgs<typename P::V, M> e = {};
     fill_axis(a.tab, e.y);
     fill_axis(a.dims == 2 ? a.tabx : a.tab, e.x);
+    if constexpr (std::is_same<P, F32>::value) {
+        fill_axis(a.tab, e.y64);
+        fill_axis(a.dims == 2 ? a.tabx : a.tab, e.x64);
+    }
     e.rho = rho;
     e.u[0] = ux;
     e.u[1] = a.dims >= 2 ? uy : nullptr;
@@ -289,7 +297,7 @@ cudaError_t launch_eq(const AuxArgs &a, void *f, const double *rho, const double
     e.pitch = a.pitch;
     e.dims = a.dims;
     e.plane = a.plane;
-    k_equilibrium<P><<<(e.nodes + 31) / 32, 32 * EQ_WARPS, 0, s>>>(e);
+    k_equilibrium<P, M><<<(e.nodes + 31) / 32, 32 * EQ_WARPS, 0, s>>>(e);
     return cudaGetLastError();
 }
 
@@ -299,6 +307,10 @@ cudaError_t glbm_launch_set_equilibrium(const AuxArgs &a, void *f, const double 
                                         const double *ux, const double *uy, const double *uz,
                                         cudaStream_t s)
 {
-    return a.prec == GLBM_FP64 ? launch_eq<F64>(a, f, rho, ux, uy, uz, s)
-                               : launch_eq<F32>(a, f, rho, ux, uy, uz, s);
+    const bool hi = a.N > GLBM_MAXN_2N1;
+    if (a.prec == GLBM_FP64)
+        return hi ? launch_eq<F64, GLBM_MAXN>(a, f, rho, ux, uy, uz, s)
+                  : launch_eq<F64, GLBM_MAXN_2N1>(a, f, rho, ux, uy, uz, s);
+    return hi ? launch_eq<F32, GLBM_MAXN>(a, f, rho, ux, uy, uz, s)
+              : launch_eq<F32, GLBM_MAXN_2N1>(a, f, rho, ux, uy, uz, s);
 }

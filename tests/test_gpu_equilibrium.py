@@ -1,7 +1,6 @@
 """The initial equilibrium (float-pair arithmetic in FP32 deviations) against the
 oracle's: a stored deviation is the exact one rounded once, so it differs from the
-oracle's FP64 value by at most half a float ulp of the deviation (2^-24 of it, with
-1 % for the pairs' own 2^-46) plus the FP64 roundings of f and of the oracle's
+oracle's FP64 value by at most half a float ulp of the deviation (2^-24 of it) plus the FP64 roundings of f and of the oracle's
 factorial sums (1e-14 of the largest population); FP64 storage by the latter alone.
 Every lattice kind, 1D to 3D, ragged sizes, the rest state exactly, and fields
 beyond the pairs' range."""
@@ -43,7 +42,7 @@ def _check(cfg, prec, amp=0.05, edit=None):
     W = o.equilibrium(one, *[zero] * d)
     tol = 1e-14 * np.abs(want).max(axis=0)
     if prec == glbm.FP32_DEV:
-        tol = tol + 1.01 * 2.0 ** -24 * np.abs(want - W) + 1e-45
+        tol = tol + 2.0 ** -24 * np.abs(want - W) + 1e-45
     assert (np.abs(got - want) <= tol).all(), float((np.abs(got - want) - tol).max())
     assert np.abs(rest - W).max() < 1e-15  # the rest state of a new context
     lat.set_equilibrium(0, one, *[zero] * d)
@@ -76,6 +75,29 @@ def test_fields_beyond_the_float_pairs(prec):
         f[0][0, 0], f[1][0, 1], f[2][1, 1] = 3e19, 1e-25, -1e-30
         f[0][2, 2], f[1][2, 2] = 1e-19, 0.0
     _check(dict(dims=2, nx=9, ny=4, k=2), prec, edit=edit)
+
+
+def test_float_pairs_round_like_fp64():
+    """The stored deviations are the FP64 formula's, rounded: against the deviations
+    of an FP64 context (E^x A there, so equal up to the rounding of its f ~ W) no
+    stored float may be further than half an ulp plus 2^-50 W."""
+    nx, ny, k = 700, 300, 3
+    rng = np.random.default_rng(11)
+    fields = [1 + 0.03 * rng.standard_normal((ny, nx))] + \
+        [0.04 * rng.standard_normal((ny, nx)) for _ in range(2)]
+    a = glbm.Lattice(dict(dims=2, nx=nx, ny=ny, k=k, tau=0.9, prec=glbm.FP32_DEV))
+    b = glbm.Lattice(dict(dims=2, nx=nx, ny=ny, k=k, tau=0.9, prec=glbm.FP64))
+    W = b.get_populations(0)
+    for lat in (a, b):
+        lat.set_equilibrium(0, *fields)
+    stored = np.empty((81, ny, nx), np.float32)
+    a.pack_columns(0, 0, nx, stored)
+    d = b.get_populations(0) - W
+    s = stored.astype(np.float64)
+    ulp = np.spacing(np.abs(stored)).astype(np.float64)
+    assert (np.abs(s - d) <= 0.5 * ulp + 2.0 ** -50 * W).all()
+    a.close()
+    b.close()
 
 
 def test_infinite_and_nan_fields_stay_in_their_node():
