@@ -565,7 +565,7 @@ static glbm_status finish_create(glbm_ctx *c, const glbm_config *cfgs, int n, vo
     if (st != GLBM_OK) return st;
     for (int i = 0; i < n; ++i) {
         CUDA_TRY(glbm_launch_set_equilibrium(aux_args(c, i), inst_ptr(c, 0, i), nullptr, nullptr,
-                                             nullptr, nullptr, c->stream));
+                                             nullptr, nullptr, nullptr, c->stream));
         c->launches += 1;
     }
     CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -792,10 +792,10 @@ static glbm_status set_equilibrium_impl(glbm_ctx *c, int inst, const double *rho
         if (uz) dw = c->d_stage + 3 * nodes;
     }
     CUDA_TRY(glbm_launch_set_equilibrium(aux_args(c, inst), inst_ptr(c, c->cur, inst), dr, du, dv, dw,
-                                         c->stream));
+                                         c->d_status, c->stream));
     c->launches += 1;
-    CUDA_TRY(set_clock(c, 0));
-    CUDA_TRY(clear_unstable(c));
+    c->t = 0;
+    c->halted = false;
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(c->stream));  // host buffers reusable on return
     return GLBM_OK;
 }
@@ -827,10 +827,11 @@ extern "C" glbm_status glbm_set_populations(glbm_ctx *c, int inst, const double 
         CUDA_TRY(cudaMemcpyAsync(c->d_stage, f, n * 8, cudaMemcpyHostToDevice, c->stream));
         src = c->d_stage;
     }
-    CUDA_TRY(glbm_launch_set_populations(aux_args(c, inst), inst_ptr(c, c->cur, inst), src, c->stream));
+    CUDA_TRY(glbm_launch_set_populations(aux_args(c, inst), inst_ptr(c, c->cur, inst), src, c->d_status,
+                                         c->stream));
     c->launches += 1;
-    CUDA_TRY(set_clock(c, 0));
-    CUDA_TRY(clear_unstable(c));
+    c->t = 0;
+    c->halted = false;
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(c->stream));
     return GLBM_OK;
 }

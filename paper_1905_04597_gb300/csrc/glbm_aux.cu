@@ -37,8 +37,9 @@ constexpr int COPY_ROWS = 8;
 
 template <typename T, bool SET>
 __global__ void __launch_bounds__(128)
-    k_copy_populations(const __grid_constant__ AuxArgs a, T *f, double *p)
+    k_copy_populations(const __grid_constant__ AuxArgs a, T *f, double *p, unsigned *status)
 {
+    if (SET && blockIdx.x + blockIdx.y + blockIdx.z + threadIdx.x == 0) reset_status(status);
     const int x = blockIdx.x * 128 + threadIdx.x, q = blockIdx.z;
     if (x >= a.Lx) return;
     const int rows = a.Ly * a.Lz, y0 = blockIdx.y * COPY_ROWS;
@@ -362,24 +363,26 @@ static int velocities(const AuxArgs &a)
 }
 
 template <bool SET>
-static cudaError_t copy_populations(const AuxArgs &a, void *f, double *p, cudaStream_t s)
+static cudaError_t copy_populations(const AuxArgs &a, void *f, double *p, unsigned *status,
+                                    cudaStream_t s)
 {
     const dim3 grid((a.Lx + 127) / 128, (a.Ly * a.Lz + COPY_ROWS - 1) / COPY_ROWS, velocities(a));
     if (a.prec == GLBM_FP64)
-        k_copy_populations<double, SET><<<grid, 128, 0, s>>>(a, static_cast<double *>(f), p);
+        k_copy_populations<double, SET><<<grid, 128, 0, s>>>(a, static_cast<double *>(f), p, status);
     else
-        k_copy_populations<float, SET><<<grid, 128, 0, s>>>(a, static_cast<float *>(f), p);
+        k_copy_populations<float, SET><<<grid, 128, 0, s>>>(a, static_cast<float *>(f), p, status);
     return cudaGetLastError();
 }
 
-cudaError_t glbm_launch_set_populations(const AuxArgs &a, void *f, const double *src, cudaStream_t s)
+cudaError_t glbm_launch_set_populations(const AuxArgs &a, void *f, const double *src,
+                                        unsigned *status, cudaStream_t s)
 {
-    return copy_populations<true>(a, f, const_cast<double *>(src), s);
+    return copy_populations<true>(a, f, const_cast<double *>(src), status, s);
 }
 
 cudaError_t glbm_launch_get_populations(const AuxArgs &a, const void *f, double *dst, cudaStream_t s)
 {
-    return copy_populations<false>(a, const_cast<void *>(f), dst, s);
+    return copy_populations<false>(a, const_cast<void *>(f), dst, nullptr, s);
 }
 
 cudaError_t glbm_launch_moments1d(const AuxArgs &a, const void *f, const MomPtrs &out,

@@ -54,6 +54,15 @@ __device__ __forceinline__ bool step_halted(const unsigned *status)
     return __ldcg(status + ST_HALT) != 0u;
 }
 
+// A new state's status words, written by one thread of the kernel that sets it (a copy
+// and two memsets of their own took longer than the words): step clock 0, no failure.
+__device__ __forceinline__ void reset_status(unsigned *status)
+{
+    status[ST_CLOCK] = 0u;
+    status[ST_FLAGS] = 0u;
+    status[ST_HALT] = 0u;
+}
+
 // Called by every CTA of a step's last launch: the last CTA to finish advances
 // the launch counter that seeds the FP32 dither of the next step (every CTA
 // read it before finishing) and the count of completed steps, and sets the

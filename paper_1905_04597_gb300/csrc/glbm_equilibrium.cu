@@ -91,6 +91,7 @@ struct EqArgs {
     std::conditional_t<std::is_same<V, df>::value, EqAxis<double, M>, NoAxis> y64, x64;
     const double *rho, *u[3];  // null: 1, 0
     void *f;
+    unsigned *status;           // the status words a new state resets, or null
     int Lx, nodes, pitch, dims;
     long long plane;
 };
@@ -173,6 +174,7 @@ __global__ void __launch_bounds__(32 * EQ_WARPS)
     __shared__ V in[5][32];                  // u_x, u_y, u_z, rho, rho - 1
     __shared__ V dx[2 * GLBM_MAXN_2N1 + 2][32];  // FP32: E^x - W^x; FP64: E^x
     __shared__ V dy[2 * M + 2][32], dz[2 * GLBM_MAXN_3D + 1][32];
+    if (a.status && blockIdx.x == 0 && threadIdx.x == 0) reset_status(a.status);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int n = blockIdx.x * 32 + lane, nc = n < a.nodes ? n : a.nodes - 1;
     const int row = nc / a.Lx, x = nc - row * a.Lx;
@@ -278,7 +280,7 @@ void fill_axis(const AxisTableHi &t, EqAxis<V, M> &e)
 
 template <class P, int M>
 cudaError_t launch_eq(const AuxArgs &a, void *f, const double *rho, const double *ux,
-                      const double *uy, const double *uz, cudaStream_t s)
+                      const double *uy, const double *uz, unsigned *status, cudaStream_t s)
 {
     EqArgs<typename P::V, M> e = {};
     fill_axis(a.tab, e.y);
@@ -292,6 +294,7 @@ cudaError_t launch_eq(const AuxArgs &a, void *f, const double *rho, const double
     e.u[1] = a.dims >= 2 ? uy : nullptr;
     e.u[2] = a.dims == 3 ? uz : nullptr;
     e.f = f;
+    e.status = status;
     e.Lx = a.Lx;
     e.nodes = a.Lx * a.Ly * a.Lz;
     e.pitch = a.pitch;
@@ -305,12 +308,12 @@ cudaError_t launch_eq(const AuxArgs &a, void *f, const double *rho, const double
 
 cudaError_t glbm_launch_set_equilibrium(const AuxArgs &a, void *f, const double *rho,
                                         const double *ux, const double *uy, const double *uz,
-                                        cudaStream_t s)
+                                        unsigned *status, cudaStream_t s)
 {
     const bool hi = a.N > GLBM_MAXN_2N1;
     if (a.prec == GLBM_FP64)
-        return hi ? launch_eq<F64, GLBM_MAXN>(a, f, rho, ux, uy, uz, s)
-                  : launch_eq<F64, GLBM_MAXN_2N1>(a, f, rho, ux, uy, uz, s);
-    return hi ? launch_eq<F32, GLBM_MAXN>(a, f, rho, ux, uy, uz, s)
-              : launch_eq<F32, GLBM_MAXN_2N1>(a, f, rho, ux, uy, uz, s);
+        return hi ? launch_eq<F64, GLBM_MAXN>(a, f, rho, ux, uy, uz, status, s)
+                  : launch_eq<F64, GLBM_MAXN_2N1>(a, f, rho, ux, uy, uz, status, s);
+    return hi ? launch_eq<F32, GLBM_MAXN>(a, f, rho, ux, uy, uz, status, s)
+              : launch_eq<F32, GLBM_MAXN_2N1>(a, f, rho, ux, uy, uz, status, s);
 }

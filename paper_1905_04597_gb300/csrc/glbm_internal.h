@@ -305,12 +305,13 @@ struct AuxArgs {
     int Lz;               // nodes along z (3D; 1 otherwise)
 };
 // Equilibrium of the fields rho (null: 1) and u_x, u_y, u_z (null: 0) of one
-// instance (glbm_equilibrium.cu; f: its populations).
+// instance (glbm_equilibrium.cu; f: its populations); with status words the launch
+// resets them for the new state (reset_status).
 cudaError_t glbm_launch_set_equilibrium(const AuxArgs &a, void *f, const double *rho,
                                         const double *ux, const double *uy, const double *uz,
-                                        cudaStream_t s);
+                                        unsigned *status, cudaStream_t s);
 cudaError_t glbm_launch_set_populations(const AuxArgs &a, void *f, const double *src,
-                                        cudaStream_t s);
+                                        unsigned *status, cudaStream_t s);
 cudaError_t glbm_launch_get_populations(const AuxArgs &a, const void *f, double *dst,
                                         cudaStream_t s);
 // Destinations of the moment fields, by the bit of GLBM_M_*; null: not wanted.
