@@ -119,6 +119,7 @@ struct glbm_ctx {
     DevAlloc A{};
     cudaStream_t stream = nullptr;
     cudaStream_t cap = nullptr;  // private stream used only for graph capture
+    SideStreams side = {};       // a batch's concurrent levels
     long long pool_elems = 0;    // elements per buffer
     void *buf[2] = {nullptr, nullptr};
     int cur = 0;                 // buffer holding X_t
@@ -393,6 +394,21 @@ static void destroy_resources(glbm_ctx *c)
     dev_free(c->A, c->d_tabs, c->stream);
     if (c->h_status) cudaFreeHost(c->h_status);
     if (c->cap) cudaStreamDestroy(c->cap);
+    if (c->side.fork) cudaEventDestroy(c->side.fork);
+    for (int k = 0; k < GLBM_SIDE_STREAMS; ++k) {
+        if (c->side.join[k]) cudaEventDestroy(c->side.join[k]);
+        if (c->side.s[k]) cudaStreamDestroy(c->side.s[k]);
+    }
+}
+
+static glbm_status create_side_streams(glbm_ctx *c)
+{
+    CUDA_TRY(cudaEventCreateWithFlags(&c->side.fork, cudaEventDisableTiming));
+    for (int k = 0; k < GLBM_SIDE_STREAMS; ++k) {
+        CUDA_TRY(cudaEventCreateWithFlags(&c->side.join[k], cudaEventDisableTiming));
+        CUDA_TRY(cudaStreamCreateWithFlags(&c->side.s[k], cudaStreamNonBlocking));
+    }
+    return GLBM_OK;
 }
 
 // Arguments of the auxiliary kernels for one instance: the pool pointer is
@@ -721,6 +737,7 @@ extern "C" glbm_status glbm_batch_create(const glbm_config *cfgs, int n, void *s
     c->tile[6] = 2;
     c->tile[7] = 1;
     glbm_status st = finish_create(c, cfgs, n, stream);
+    if (st == GLBM_OK) st = create_side_streams(c);
     if (st == GLBM_OK) st = build_items(c);
     if (st != GLBM_OK) {
         destroy_resources(c);
@@ -1022,7 +1039,7 @@ static bool df_eligible(const glbm_ctx *c)
 static cudaError_t launch_step(const glbm_ctx *c, const void *fin, void *fout, cudaStream_t s,
                                int node = -1)
 {
-    if (c->hetero) return glbm_launch_batched_f32(batch_args(c, fin, fout), s);
+    if (c->hetero) return glbm_launch_batched_f32(batch_args(c, fin, fout), s, c->side);
     const int N = c->geo[0].N;
     if (c->small) return launch_small(c, fin, fout, s);
     if (c->dims == 3)

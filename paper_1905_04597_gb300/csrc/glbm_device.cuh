@@ -68,11 +68,12 @@ __device__ __forceinline__ void reset_status(unsigned *status)
 // read it before finishing) and the count of completed steps, and sets the
 // halt word when a node of this or an earlier step left the positivity
 // domain (flag_unstable fences each flag before its CTA reaches the count).
-__device__ __forceinline__ void finish_step(unsigned *status)
+// `total`: the CTAs of the step (its launch's, or those of a batch's concurrent
+// launches).
+__device__ __forceinline__ void finish_step(unsigned *status, unsigned total)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
-        const unsigned total = gridDim.x * gridDim.y * gridDim.z;
         if (atomicAdd(status + ST_DONE, 1u) == total - 1u) {
             status[ST_DONE] = 0u;
             atomicAdd(status + ST_CLOCK, 1u);
@@ -80,6 +81,11 @@ __device__ __forceinline__ void finish_step(unsigned *status)
             if (atomicOr(status + ST_FLAGS, 0u) & 1u) atomicExch(status + ST_HALT, 1u);
         }
     }
+}
+
+__device__ __forceinline__ void finish_step(unsigned *status)
+{
+    finish_step(status, gridDim.x * gridDim.y * gridDim.z);
 }
 
 // Load of a population by the step tiles: an ordinary (weak, L1-cached) load,

@@ -218,10 +218,26 @@ struct BatchArgs {
     int shape[GLBM_MAXN + 1];  // FP32 tile shape index of each level
     unsigned *status, *step_ctr, *done_ctr;
 };
+// The same for one level's launch.
+struct BatchLevelArgs {
+    AxisTable tab;
+    const void *fin;
+    void *fout;
+    const InstParams *ip;
+    const int4 *items;         // this level's
+    unsigned *status, *step_ctr;
+    unsigned total;            // CTAs of the whole step, or 0: the launch is not a step
+};
+// Two streams beside a context's own, and the events that fork and join them.
+constexpr int GLBM_SIDE_STREAMS = 2;
+struct SideStreams {
+    cudaStream_t s[GLBM_SIDE_STREAMS];
+    cudaEvent_t fork, join[GLBM_SIDE_STREAMS];
+};
 int glbm_batched_launches(const BatchArgs &a);  // launches per step (levels present)
-cudaError_t glbm_launch_batched_f32(const BatchArgs &a, cudaStream_t s);
+cudaError_t glbm_launch_batched_f32(const BatchArgs &a, cudaStream_t s, const SideStreams &side);
 cudaError_t glbm_launch_batched_level(int N, const BatchArgs &a, bool advance, cudaStream_t s);
-// One level's launch of a batch step; `advance` moves the launch counter on.
+// One level's launch of a batch step; `advance`: it counts towards the step's end.
 template <int N>
 cudaError_t glbm_batched_level(const BatchArgs &a, bool advance, cudaStream_t s);
 
