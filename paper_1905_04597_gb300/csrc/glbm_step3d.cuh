@@ -37,6 +37,8 @@ struct Step3D {
 
     struct Smem {
         T part[R][G][8][32];  // (s, c) of delta rho, j_x, j_y, j_z per row and group
+        T tot[R][8][32];      // and over the groups
+        T dev[R][3][Q1][32];  // E - W of the nodes per axis (FP64: E^x on the x axis)
         T rw[2][32];          // wall density (FP64) or its deviation (FP32): lo, hi
         T dsum[NV][2][32];
     };
@@ -163,8 +165,19 @@ struct Step3D {
                 if (nz != 0) acc2(s_z, c_z, mul_rn(T(nz), rs));
             }
         }
-        {
-            T *pp = &sm.part[r][g][0][lane];
+        // ---- phase 2: moments, equilibrium, relaxation, store --------------
+        // The G warps of a node share this work: warp f sums functional f over the
+        // groups, then warp a takes the velocity of axis a and its equilibrium
+        // polynomials; the values meet in shared memory. Every warp for itself took
+        // 250 of the 1370 instructions of a thread at D3Q125, where the issue slots
+        // bound the kernel (IPC 3.1): 250 x 61 x 45 FP32 160 -> 143 us per step, 256 x
+        // 64 x 32 FP64 1203 -> 933 us (GB300).
+        T tS[4], tC[4];  // delta rho (FP64: rho), j_x, j_y, j_z: sums and compensations
+        if constexpr (G == 1) {
+            tS[0] = s_r, tS[1] = s_x, tS[2] = s_y, tS[3] = s_z;
+            tC[0] = c_r, tC[1] = c_x, tC[2] = c_y, tC[3] = c_z;
+        } else {
+            T *const pp = &sm.part[r][g][0][lane];
             pp[0 * 32] = s_r;
             pp[1 * 32] = c_r;
             pp[2 * 32] = s_x;
@@ -173,70 +186,72 @@ struct Step3D {
             pp[5 * 32] = c_y;
             pp[6 * 32] = s_z;
             pp[7 * 32] = c_z;
-        }
-        __syncthreads();
-
-        // ---- phase 2: moments, equilibrium, relaxation, store --------------
-        T S_r = T(0), C_r = T(0), S_x = T(0), C_x = T(0), S_y = T(0), C_y = T(0), S_z = T(0),
-          C_z = T(0);
+            __syncthreads();
+            for (int q = g; q < 4; q += G) {
+                T S = T(0), C = T(0);
 #pragma unroll
-        for (int gi = 0; gi < G; ++gi) {
-            const T *pp = &sm.part[r][gi][0][lane];
-            acc2(S_r, C_r, pp[0 * 32]);
-            acc2(S_x, C_x, pp[2 * 32]);
-            acc2(S_y, C_y, pp[4 * 32]);
-            acc2(S_z, C_z, pp[6 * 32]);
-            if (DEV) {
-                C_r += pp[1 * 32];
-                C_x += pp[3 * 32];
-                C_y += pp[5 * 32];
-                C_z += pp[7 * 32];
+                for (int gi = 0; gi < G; ++gi) {
+                    acc2(S, C, sm.part[r][gi][2 * q][lane]);
+                    if (DEV) C += sm.part[r][gi][2 * q + 1][lane];
+                }
+                sm.tot[r][2 * q][lane] = S;
+                if (DEV) sm.tot[r][2 * q + 1][lane] = C;
             }
+            __syncthreads();
+            tS[0] = sm.tot[r][0][lane];
+            tC[0] = DEV ? sm.tot[r][1][lane] : T(0);
         }
-        const T m0 = S_r + C_r;
+        const T m0 = DEV ? tS[0] + tC[0] : tS[0];
         const T rho = DEV ? T(1) + m0 : m0;
         const T drho = DEV ? m0 : m0 - T(1);
-        const T inv_rho = T(1) / rho;
-        const T jx = S_x + C_x, jy = S_y + C_y, jz = S_z + C_z;
-        T ux = jx * inv_rho, uy = jy * inv_rho, uz = jz * inv_rho;
         const unsigned hnode = DEV ? hash32((unsigned)((z * Ly + y) * Lx + x) ^ seed) : 0u;
-        if constexpr (DEV) {
-            // u = j / (1 + delta rho), rounded stochastically (as in the 2D tile):
-            // j times the rounded reciprocal alone carries a fixed relative bias
-            // of up to 2^-24 where rho lies just below 1
-            const T dux = dither_ulp(ux, dither_unit(dither_word_ux(hnode)));
-            const T duy = dither_ulp(uy, dither_unit(dither_word_uy(hnode)));
-            const T duz = dither_ulp(uz, dither_unit(dither_word_uz(hnode)));
-            ux = fma(fma(-ux, drho, (S_x - ux) + C_x) + dux, inv_rho, ux);
-            uy = fma(fma(-uy, drho, (S_y - uy) + C_y) + duy, inv_rho, uy);
-            uz = fma(fma(-uz, drho, (S_z - uz) + C_z) + duz, inv_rho, uz);
-        }
-        if (active) {
-            const T umax = (T)(0.816496580927726 * N);  // sqrt(2/3) N (Sec. 3)
-            if (!(rho > T(0)) || !(fabs(ux) <= umax) || !(fabs(uy) <= umax) || !(fabs(uz) <= umax))
-                flag_unstable(status);
-        }
-        T dx[Q1], dy[Q1], dz[Q1];
-        if constexpr (DEV) {
-            // polynomial values rounded stochastically, one draw per node and axis
-            eq_dev_all_sr<N>(tab, ux, dither_unit2(dither_word_ex(hnode)), dx);
-            eq_dev_all_sr<N>(tab, uy, dither_unit2(dither_word_ey(hnode)), dy);
-            eq_dev_all_sr<N>(tab, uz, dither_unit2(dither_word_ez(hnode)), dz);
-        } else {
-            eq_dev_all<N, T>(tab, ux, dx);
-            eq_dev_all<N, T>(tab, uy, dy);
-            eq_dev_all<N, T>(tab, uz, dz);
+        const T inv_rho = G == 1 || g < 3 ? T(1) / rho : T(0);
+        for (int ax = G == 1 ? 0 : g; ax < 3; ax += G) {
+            T S, C;
+            if constexpr (G == 1) {
+                S = ax == 0 ? tS[1] : ax == 1 ? tS[2] : tS[3];
+                C = ax == 0 ? tC[1] : ax == 1 ? tC[2] : tC[3];
+            } else {
+                S = sm.tot[r][2 + 2 * ax][lane];
+                C = DEV ? sm.tot[r][3 + 2 * ax][lane] : T(0);
+            }
+            T u = (DEV ? S + C : S) * inv_rho;
+            float re = 0.0f;
+            if constexpr (DEV) {
+                // u = j / (1 + delta rho), rounded stochastically (as in the 2D tile):
+                // j times the rounded reciprocal alone carries a fixed relative bias
+                // of up to 2^-24 where rho lies just below 1; the polynomial values
+                // are rounded stochastically too, one draw per node and axis
+                const unsigned wu = ax == 0   ? dither_word_ux(hnode)
+                                    : ax == 1 ? dither_word_uy(hnode)
+                                              : dither_word_uz(hnode);
+                const unsigned we = ax == 0   ? dither_word_ex(hnode)
+                                    : ax == 1 ? dither_word_ey(hnode)
+                                              : dither_word_ez(hnode);
+                const T du = dither_ulp(u, dither_unit(wu));
+                u = fma(fma(-u, drho, (S - u) + C) + du, inv_rho, u);
+                re = dither_unit2(we);
+            }
+            if (active) {
+                const T umax = (T)(0.816496580927726 * N);  // sqrt(2/3) N (Sec. 3)
+                if (!(rho > T(0)) || !(fabs(u) <= umax)) flag_unstable(status);
+            }
+            T d[Q1];
+            if constexpr (DEV)
+                eq_dev_all_sr<N>(tab, u, re, d);
+            else
+                eq_dev_all<N, T>(tab, u, d);
 #pragma unroll
-            for (int ix = 0; ix < Q1; ++ix) dx[ix] += A::W(tab, ix);  // E^x, once per node
+            for (int i = 0; i < Q1; ++i) {
+                if (!DEV && ax == 0) d[i] += A::W(tab, i);  // E^x, once per node
+                sm.dev[r][ax][i][lane] = d[i];
+            }
         }
-
-        // ZROW: this thread's n_y deviation, selected once
-        T dy_g = dy[0];
-        if constexpr (ZROW) {
+        if constexpr (G > 1) __syncthreads();
+        T dx[Q1];
 #pragma unroll
-            for (int i = 1; i < Q1; ++i)
-                if (g == i) dy_g = dy[i];
-        }
+        for (int ix = 0; ix < Q1; ++ix) dx[ix] = sm.dev[r][0][ix][lane];
+        const T dy_g = ZROW ? sm.dev[r][1][g][lane] : T(0);  // ZROW: this thread's n_y
         const T om = DEV ? (T)ip.omega_f : (T)ip.omega;
         const T gto = DEV ? (T)ip.g_theta_om_f : (T)ip.g_theta_om;  // g / (theta omega)
         if (!live) return;  // an earlier step halted the run: store nothing
@@ -251,20 +266,7 @@ struct Step3D {
             if (row < NROW) {
                 const int iz = row_z(row, k), iy = row_y(row, g);
                 const T wy = A::W(tab, iy), wz = A::W(tab, iz);
-                // runtime row: the per-axis deviations by a select chain
-                T dyv, dzv;
-                if constexpr (ZROW) {
-                    dzv = dz[k];
-                    dyv = dy_g;
-                } else {
-                    dyv = dy[0];
-                    dzv = dz[0];
-#pragma unroll
-                    for (int i = 1; i < Q1; ++i) {
-                        if (iy == i) dyv = dy[i];
-                        if (iz == i) dzv = dz[i];
-                    }
-                }
+                const T dyv = ZROW ? dy_g : sm.dev[r][1][iy][lane], dzv = sm.dev[r][2][iz][lane];
                 const T rez = rho * (wz + dzv);       // rho e^z
                 const T rez_y = rez * (wy + dyv);     // rho e^y e^z
                 const T wyz = mul_rn(wy, wz);
@@ -327,7 +329,7 @@ struct Step3D {
                         // dx holds E^x itself in FP64 mode; f^eq - f0 in one
                         // fused rounding, the force term, f0 + omega (...)
                         T d = fma(dx[ix], rez_y, -f0);
-                        if (nx != 0) d = fma(A::WN(tab, ix), gr, d);
+                        if (nx != 0 && gto != T(0)) d = fma(A::WN(tab, ix), gr, d);
                         v = fma(om, d, f0);
                     }
                     op[ix * plane] = v;
