@@ -20,6 +20,7 @@
 namespace {
 
 constexpr int RUN1D_THREADS = 512;
+constexpr int RUN1D_SMEM = 200 * 1024;
 
 __device__ __forceinline__ void cluster_sync_all()
 {
@@ -202,8 +203,10 @@ cudaError_t launch_n(Run1DArgs &r, int n_inst, cudaStream_t s, int *ok)
         const int H = N * r.m;
         if (H > L / C) return cudaSuccess;  // shorter than the reach: the caller's other paths
         const size_t smem = sizeof(T) * Q1 * (2 * (size_t)(r.maxn + 2 * H) + 4 * (size_t)H);
-        if (smem > 200 * 1024) return cudaSuccess;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (smem > RUN1D_SMEM) return cudaSuccess;
+        // (one limit for every launch: a smaller one set by another thread in between
+        // would refuse this one)
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RUN1D_SMEM);
         if (e == cudaSuccess && C > 8)
             e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;

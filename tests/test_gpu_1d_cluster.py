@@ -88,3 +88,20 @@ def test_failing_step_inside_a_call(prec):
     np.testing.assert_array_equal(a.get_populations(0), b.get_populations(0))
     a.close()
     b.close()
+
+
+def test_calls_longer_than_one_launch():
+    """A call of more steps than one launch takes equals the same steps in two calls."""
+    cfg = dict(dims=1, nx=64, k=0, tau=0.8, prec=glbm.FP32_DEV)
+    a, b = glbm.Lattice(cfg), glbm.Lattice(cfg)
+    x = np.arange(64) / 64
+    for lat in (a, b):
+        lat.set_equilibrium(0, 1 + 0.05 * np.sin(2 * np.pi * x), np.zeros(64))
+    n0 = a.kernel_launches
+    a.step(65536 + 37)
+    assert a.kernel_launches - n0 == 2 and a.time == 65536 + 37
+    b.step(40000)
+    b.step(25536 + 37)
+    np.testing.assert_array_equal(a.get_populations(0), b.get_populations(0))
+    a.close()
+    b.close()
