@@ -101,8 +101,12 @@ __device__ __forceinline__ T ld_pop(const T *p)
 
 // ---- dataflow stepping (GLBM_DF_CHUNK, glbm_internal.h) -------------------
 
-// Let the next launch of the stream start its CTAs now (their waits below
-// keep them off data that is not ready).
+// Let the next launch of the stream start its CTAs now (their waits keep them off
+// data that is not ready). A small launch that prepares wall sums for the main one
+// behind it waits for the work before both first and lets the main launch start next:
+// from then on everything older than the small launch is complete, and the main
+// launch waits only where it needs the sums (in at least one CTA, so that its own
+// completion implies the small launch's).
 __device__ __forceinline__ void df_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
@@ -524,19 +528,25 @@ inline bool programmatic(const Args &)
     return true;
 }
 
-template <typename Args>
-inline cudaError_t launch_serialized(void (*kern)(Args), dim3 grid, dim3 block, cudaStream_t s,
-                                     const Args &a)
+template <typename... Params, typename Args, typename... More>
+inline cudaError_t launch_serialized_smem(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem,
+                                          cudaStream_t s, const Args &a, const More &...more)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = programmatic(a) ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, a);
+    return cudaLaunchKernelEx(&cfg, kern, a, more...);
+}
+template <typename... Params, typename Args, typename... More>
+inline cudaError_t launch_serialized(void (*kern)(Params...), dim3 grid, dim3 block, cudaStream_t s,
+                                     const Args &a, const More &...more)
+{
+    return launch_serialized_smem(kern, grid, block, 0, s, a, more...);
 }

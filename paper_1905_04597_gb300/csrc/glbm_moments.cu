@@ -44,17 +44,9 @@ cudaError_t glbm_launch_moments(const AuxArgs &a, const void *f, double *rw, con
         const int cols = a.Lx * a.Lz, QX = ax_q(a.tabx);
         const dim3 grid((cols + WALL_TX - 1) / WALL_TX, 2), blk(WALL_TX * WALL_SL);
         const int v0 = ax_vel(a.tabx, 0), vs = a.tabx.zv ? 2 : 1;
-        if (d3) {
-            if (a.prec == GLBM_FP64)
-                k_moment_walls<3, double><<<grid, blk, 0, s>>>(m, QX, v0, vs, rw);
-            else
-                k_moment_walls<3, float><<<grid, blk, 0, s>>>(m, QX, v0, vs, rw);
-        } else if (a.prec == GLBM_FP64) {
-            k_moment_walls<2, double><<<grid, blk, 0, s>>>(m, QX, v0, vs, rw);
-        } else {
-            k_moment_walls<2, float><<<grid, blk, 0, s>>>(m, QX, v0, vs, rw);
-        }
-        const cudaError_t e = cudaGetLastError();
+        auto *const kern = d3 ? (a.prec == GLBM_FP64 ? k_moment_walls<3, double> : k_moment_walls<3, float>)
+                              : (a.prec == GLBM_FP64 ? k_moment_walls<2, double> : k_moment_walls<2, float>);
+        const cudaError_t e = launch_serialized(kern, grid, blk, s, m, QX, v0, vs, rw);
         if (e != cudaSuccess) return e;
     }
     bool full = false;  // any field beyond the density and the velocities
