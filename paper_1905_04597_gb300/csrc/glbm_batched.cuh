@@ -11,8 +11,15 @@
 #include "glbm_step2d_pair.cuh"
 #include "glbm_tiles.h"
 
+// CTAs per SM asked of a one-node tile (0: the compiler's choice). At level 7 the
+// compiler took 128 registers, three CTAs of (5, 1, 1); 96 hold its three rows of 15
+// without spills, four CTAs (GB300, 64 channels of 64 columns, per step: 283 -> 277.6
+// us).
 template <int N, int G, int R>
-__global__ void __launch_bounds__(32 * G * R)
+constexpr int ITEMS_CTAS = N == 7 && R == 1 && G == 5 ? 4 : 0;
+
+template <int N, int G, int R>
+__global__ void __launch_bounds__(32 * G * R, ITEMS_CTAS<N, G, R>)
     k_step2d_items(const __grid_constant__ BatchLevelArgs a)
 {
     using S = Step2D<N, float, G, R>;
