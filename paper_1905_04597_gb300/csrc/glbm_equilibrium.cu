@@ -13,10 +13,14 @@
 // instead: the value before the rounding to float is exact to 2^-43 of its terms, and
 // where the rounding could go either way within 2^-41 (about one population in 2^16)
 // it is formed in FP64, so every stored float is that of the FP64 formula. Fields
-// outside 1e-18..1e18 in magnitude (or not finite) take FP64. Measured on GB300, FP32:
-// D2Q81 512 x 256 95 -> 29 us, D2Q289 1024 x 128 311 -> 80 us, D3Q125 250 x 61 x 45
-// 815 -> 256 us, D1Q3 x D1Q28 200 nodes (FP64) 25 -> 10 us; large FP64 lattices stay
-// on the FP64 pipe (D2Q81 54 us).
+// outside 1e-18..1e18 in magnitude (or not finite) take FP64. The pairs' kernel is
+// bound by its issue slots (92 instructions per population at D3Q125 and 65 at D2Q289
+// with run-time row lengths), so the x axis's velocities are a template parameter,
+// populations too close to call are collected and formed after their row, and E^y,
+// rho E^z and rho (E^z - W^z) are formed once per node. Measured on GB300, FP32, FP64
+// pipe -> pairs -> this: D2Q81 512 x 256 95 -> 39 -> 33 us, D2Q289 1024 x 128 311 -> 95
+// -> 79 us, D3Q125 250 x 61 x 45 815 -> 257 -> 183 us; D1Q3 x D1Q28 200 nodes (FP64)
+// 25 -> 10 us; large FP64 lattices stay on the FP64 pipe (D2Q81 54 us).
 #include "glbm_device.cuh"
 
 namespace {
@@ -89,6 +93,9 @@ struct EqArgs {
     EqAxis<V, M> y, x;  // 3D: y holds for z too
     // float pairs: the FP64 tables too
     std::conditional_t<std::is_same<V, df>::value, EqAxis<double, M>, NoAxis> y64, x64;
+    // float pairs, 3D: W^y W^z
+    std::conditional_t<std::is_same<V, df>::value, V, NoAxis> wyz[2 * GLBM_MAXN_3D + 1]
+                                                                 [2 * GLBM_MAXN_3D + 1];
     const double *rho, *u[3];  // null: 1, 0
     void *f;
     unsigned *status;           // the status words a new state resets, or null
@@ -165,7 +172,8 @@ __device__ __forceinline__ bool eq_dev(df w, df B, df d, df A, float &out)
 
 constexpr int EQ_WARPS = 4;
 
-template <class P, int M>
+// QX: the velocities of the x axis (float pairs), or 0: known at run time only.
+template <class P, int M, int QX>
 __global__ void __launch_bounds__(32 * EQ_WARPS)
     k_equilibrium(const __grid_constant__ EqArgs<typename P::V, M> a)
 {
@@ -174,6 +182,9 @@ __global__ void __launch_bounds__(32 * EQ_WARPS)
     __shared__ V in[5][32];                  // u_x, u_y, u_z, rho, rho - 1
     __shared__ V dx[2 * GLBM_MAXN_2N1 + 2][32];  // FP32: E^x - W^x; FP64: E^x
     __shared__ V dy[2 * M + 2][32], dz[2 * GLBM_MAXN_3D + 1][32];
+    // float pairs: E^y, and (3D) rho E^z and rho (E^z - W^z)
+    __shared__ V ey[F ? 2 * M + 2 : 1][32], pz[F ? 2 * GLBM_MAXN_3D + 1 : 1][32],
+        qz[F ? 2 * GLBM_MAXN_3D + 1 : 1][32];
     if (a.status && blockIdx.x == 0 && threadIdx.x == 0) reset_status(a.status);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int n = blockIdx.x * 32 + lane, nc = n < a.nodes ? n : a.nodes - 1;
@@ -214,38 +225,63 @@ __global__ void __launch_bounds__(32 * EQ_WARPS)
             plus = P::add(tab.W[ip], plus);
             minus = P::add(tab.W[im], minus);
         }
+        if (F && ax == 1) {
+            ey[im][lane] = P::add(tab.W[im], minus);
+            ey[ip][lane] = P::add(tab.W[ip], plus);
+        }
+        if (F && ax == 2) {
+            const V r = in[3][lane];
+            pz[im][lane] = P::mul(r, P::add(tab.W[im], minus));
+            pz[ip][lane] = P::mul(r, P::add(tab.W[ip], plus));
+            qz[im][lane] = P::mul(r, minus);
+            qz[ip][lane] = P::mul(r, plus);
+            continue;
+        }
         V(*const d)[32] = ax == 0 ? dx : ax == 1 ? dy : dz;
         d[im][lane] = minus;
         d[ip][lane] = plus;
     }
     __syncthreads();
-    const int Qx = 2 * a.x.N + 1 + a.x.zv, Qy = a.dims >= 2 ? 2 * a.y.N + 1 + a.y.zv : 1;
+    const int Qx = QX ? QX : 2 * a.x.N + 1 + a.x.zv, Qy = a.dims >= 2 ? 2 * a.y.N + 1 + a.y.zv : 1;
     const int rows = a.dims == 3 ? Qy * Qy : Qy;
     const V r = in[3][lane], r1 = in[4][lane];
     const bool live = n < a.nodes, pairs = !((bad >> lane) & 1u);
-    for (int j = w; j < rows; j += EQ_WARPS) {
+    int iz = 0, iy = w;
+    for (int j = w; j < rows; j += EQ_WARPS, iy += EQ_WARPS) {
         V A = r, B = r1;
-        const int iz = a.dims == 3 ? j / Qy : 0, iy = j - iz * Qy;
-        if (a.dims >= 2) {
-            const V wy = a.y.W[iy], d = dy[iy][lane], E = P::add(wy, d);
-            if (a.dims == 2) {
-                A = P::mul(r, E);
-                if (F) B = P::fma_(r1, wy, P::mul(r, d));
+        if (a.dims == 3) {
+            for (; iy >= Qy; iy -= Qy) ++iz;
+            if constexpr (F) {
+                const V z = pz[iz][lane];
+                A = P::mul(z, ey[iy][lane]);
+                B = P::fma_(r1, a.wyz[iz][iy],
+                            P::fma_(dy[iy][lane], z, P::mul(a.y.W[iy], qz[iz][lane])));
             } else {
-                const V wz = a.y.W[iz], e = dz[iz][lane], Ez = P::add(wz, e);
-                A = P::mul(r, P::mul(E, Ez));
-                if (F) B = P::fma_(r1, P::mul(wy, wz), P::mul(r, P::fma_(d, Ez, P::mul(wy, e))));
+                A = P::mul(r, P::mul(P::add(a.y.W[iy], dy[iy][lane]), P::add(a.y.W[iz], dz[iz][lane])));
+            }
+        } else if (a.dims == 2) {
+            if constexpr (F) {
+                A = P::mul(r, ey[iy][lane]);
+                B = P::fma_(r1, a.y.W[iy], P::mul(r, dy[iy][lane]));
+            } else {
+                A = P::mul(r, P::add(a.y.W[iy], dy[iy][lane]));
             }
         }
         if (!live) continue;
         const long long o = base + (long long)(j * Qx) * a.plane;
         if constexpr (F) {
             float *out = static_cast<float *>(a.f) + o;
-#pragma unroll 3
-            for (int ix = 0; ix < Qx; ++ix, out += a.plane) {
+            unsigned open = 0u;  // columns to form in FP64
+#pragma unroll
+            for (int ix = 0; ix < QX; ++ix, out += a.plane) {
                 float v;
-                if (!(eq_dev(a.x.W[ix], B, dx[ix][lane], A, v) && pairs)) v = eq_exact(a, nc, iz, iy, ix);
+                if (!eq_dev(a.x.W[ix], B, dx[ix][lane], A, v)) open |= 1u << ix;
                 *out = v;
+            }
+            if (!pairs) open = (1u << QX) - 1u;
+            for (; open; open &= open - 1u) {
+                const int ix = __ffs(open) - 1;
+                static_cast<float *>(a.f)[o + ix * a.plane] = eq_exact(a, nc, iz, iy, ix);
             }
         } else {
             double *out = static_cast<double *>(a.f) + o;
@@ -288,6 +324,10 @@ cudaError_t launch_eq(const AuxArgs &a, void *f, const double *rho, const double
     if constexpr (std::is_same<P, F32>::value) {
         fill_axis(a.tab, e.y64);
         fill_axis(a.dims == 2 ? a.tabx : a.tab, e.x64);
+        df *const tag = nullptr;
+        for (int i = 0; a.dims == 3 && i < ax_q(a.tab); ++i)
+            for (int j = 0; j < ax_q(a.tab); ++j)
+                e.wyz[i][j] = host_value(a.tab.W[i] * a.tab.W[j], tag);
     }
     e.rho = rho;
     e.u[0] = ux;
@@ -300,7 +340,26 @@ cudaError_t launch_eq(const AuxArgs &a, void *f, const double *rho, const double
     e.pitch = a.pitch;
     e.dims = a.dims;
     e.plane = a.plane;
-    k_equilibrium<P, M><<<(e.nodes + 31) / 32, 32 * EQ_WARPS, 0, s>>>(e);
+    const int blocks = (e.nodes + 31) / 32, threads = 32 * EQ_WARPS;
+    if constexpr (std::is_same<P, F64>::value) {
+        k_equilibrium<P, M, 0><<<blocks, threads, 0, s>>>(e);
+    } else {
+        const int QX = 2 * e.x.N + 1 + e.x.zv;
+        if constexpr (M > GLBM_MAXN_2N1) {  // these levels are compiled with D1Q3 along x
+            if (QX != 3) return cudaErrorInvalidValue;
+            k_equilibrium<P, M, 3><<<blocks, threads, 0, s>>>(e);
+        } else {
+            switch (QX) {
+#define GLBM_CASE(QX) \
+            case QX: k_equilibrium<P, M, QX><<<blocks, threads, 0, s>>>(e); break;
+                GLBM_CASE(3) GLBM_CASE(4) GLBM_CASE(5) GLBM_CASE(6) GLBM_CASE(7) GLBM_CASE(8)
+                GLBM_CASE(9) GLBM_CASE(10) GLBM_CASE(11) GLBM_CASE(12) GLBM_CASE(13) GLBM_CASE(14)
+                GLBM_CASE(15) GLBM_CASE(16) GLBM_CASE(17) GLBM_CASE(18)
+#undef GLBM_CASE
+            default: return cudaErrorInvalidValue;
+            }
+        }
+    }
     return cudaGetLastError();
 }
 
