@@ -485,9 +485,10 @@ __global__ void __launch_bounds__(32 * MOM_WARPS)
     if (a.bc == GLBM_BC_WALLS) {
         wait_prior_grid();  // the wall densities
         const int vmax = a.zv ? 2 * a.N + 1 : a.N, col = z * a.Lx + x;
-        if (y < vmax) mom_emitted<DIM, DEV, FULL>(a, a.ip->kw_lo, a.rw[col], y, 1.0, m);
+        if (y < vmax) mom_emitted<DIM, DEV, FULL>(a, a.ip->kw_lo, __ldcg(a.rw + col), y, 1.0, m);
         if (a.Ly - 1 - y < vmax)
-            mom_emitted<DIM, DEV, FULL>(a, a.ip->kw_hi, a.rw[a.Lx * a.Lz + col], a.Ly - 1 - y, -1.0, m);
+            mom_emitted<DIM, DEV, FULL>(a, a.ip->kw_hi, __ldcg(a.rw + (a.Lx * a.Lz + col)), a.Ly - 1 - y,
+                                         -1.0, m);
     }
     if (n >= nodes) return;
     const double rho = m[0], jx = m[1], jy = m[2];
