@@ -216,9 +216,9 @@ size_t glbm_elem_size(const glbm_ctx *ctx);
  * and the call returns GLBM_E_UNSTABLE with "k of n steps completed" in
  * glbm_last_error(). Further glbm_step calls complete no step (k = 0) until a
  * new state is set (glbm_set_equilibrium, glbm_set_populations, glbm_load).
- * 1D contexts step their instances one after another, each stopping at its
- * own failing step; there glbm_time() advances by the fewest steps any
- * instance completed. In dataflow mode (glbm_set_dataflow; calls of 2 or more
+ * In a 1D context each instance stops at its own failing step, the instances
+ * behind a failing one keep the state of the call's start, and glbm_time()
+ * advances by the fewest steps any instance completed. In dataflow mode (glbm_set_dataflow; calls of 2 or more
  * steps) the chunks' launches overlap; the contract is the same: the call
  * writes only the other two of three state buffers (the third is allocated on
  * the first such call), so its starting state survives, and when a node fails

@@ -1299,16 +1299,32 @@ extern "C" glbm_status glbm_step(glbm_ctx *c, int64_t n)
     int64_t done = 0;  // steps of every instance completed by this call
     bool bad = false;
     if (c->dims == 1) {
-        // one instance: launches of at most 2^16 steps (24 ms at D1Q5 x 1000 in FP32),
-        // so that a run that leaves the positivity domain is known, and repeated from
-        // there, soon after
-        const int64_t most = c->n_inst > 1 ? n : (int64_t)1 << 16;
+        // launches of at most 2^16 steps (24 ms at D1Q5 x 1000 in FP32), so that a run
+        // that leaves the positivity domain is known soon after. One instance is
+        // repeated from the start of the failing launch. Several instances are repeated
+        // from the start of the call: an instance behind a failing one keeps that state,
+        // so its buffer stays out of the launches after the first (the third state buffer
+        // takes its place; without memory for it the instances step one after another)
+        const int64_t most = (int64_t)1 << 16;
+        const bool keep = c->n_inst > 1 && n > most;
         bool run = n > 0 && !c->halted;
+        if (run && keep) {
+            const glbm_status st = spare_ready(c);
+            if (st != GLBM_OK && st != GLBM_E_NOMEM) return st;
+            run = st == GLBM_OK;
+        }
+        const Binding start = binding(c);
         while (run && done < n) {
             const int64_t m = std::min<int64_t>(n - done, most);
             glbm_status st = step_1d_clusters(c, m, &run);
             if (st != GLBM_OK) return st;
-            if (run) done += m;
+            if (run) {
+                if (keep && done == 0) std::swap(c->buf[1 - c->cur], c->spare);
+                done += m;
+            } else if (keep) {
+                rebind(c, start);
+                done = 0;
+            }
         }
         if (!run) {
             // the rest, instances one after another; each stops at its own failing step
