@@ -319,12 +319,16 @@ cudaError_t launch_step1d_t(const AuxArgs &a, const void *fin, void *fout, int i
     return cudaGetLastError();
 }
 
+constexpr int RESIDENT_SMEM = 200 * 1024;
+
 template <int N, typename T>
 cudaError_t launch_resident_n(const AuxArgs &a, T *f, int inst, long long steps,
                               unsigned *status, cudaStream_t s, size_t smem)
 {
+    // (one limit for every launch: a smaller one set by another thread in between
+    // would refuse this one)
     cudaError_t e = cudaFuncSetAttribute(k_run1d_resident<N, T>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, RESIDENT_SMEM);
     if (e != cudaSuccess) return e;
     cudaFuncAttributes fa;  // FP64 of the higher levels: fewer threads than 1024 fit
     e = cudaFuncGetAttributes(&fa, k_run1d_resident<N, T>);
@@ -341,7 +345,7 @@ cudaError_t launch_resident_t(const AuxArgs &a, void *fv, int inst, long long st
 {
     const size_t smem = (size_t)2 * (2 * a.N + 1) * a.Lx * sizeof(T);
     *ok = 0;
-    if (smem > 200 * 1024) return cudaSuccess;  // caller falls back to per-step launches
+    if (smem > RESIDENT_SMEM) return cudaSuccess;  // caller falls back to per-step launches
     *ok = 1;
     T *f = static_cast<T *>(fv) + (long long)inst * a.inst_stride;
     switch (a.N) {

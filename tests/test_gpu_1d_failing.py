@@ -94,3 +94,36 @@ def test_long_call_through_three_buffers():
         np.testing.assert_array_equal(lat.get_populations(i), one.get_populations(0))
         one.close()
     lat.close()
+
+
+def test_two_threads_with_lattices_of_different_size():
+    """The repeat of failing runs in one CTA sets its kernel's shared-memory limit: a
+    small lattice in one thread must not refuse the launch of a large one in another."""
+    import threading
+
+    import torch
+    errors = []
+
+    def work(L):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                lat = glbm.Lattice(dict(dims=1, nx=L, k=0, tau=0.02))
+                rho = torch.where(torch.arange(L, device="cuda") < L // 2, 1.0, 0.01).double()
+                u = torch.zeros(L, dtype=torch.float64, device="cuda")
+                for _ in range(2000):
+                    lat.set_equilibrium(0, rho, u)
+                    try:
+                        lat.step(40)
+                        errors.append("no failure")
+                    except glbm.UnstableError:
+                        pass
+                lat.close()
+        except Exception as e:
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=(L,)) for L in (40, 2000)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[:3]
