@@ -148,6 +148,7 @@ struct glbm_ctx {
     long long df_words = 0;
     void *spare = nullptr;         // third state buffer of dataflow calls (allocated on first use)
     bool halted = false;           // a glbm_step stopped at a failing step (until a new state)
+    Run1DPlan run1d = {};          // 1D: how its lattices step on clusters
     int64_t t = 0;
     int64_t launches = 0;
     unsigned clock_word = 0;  // host copy uploaded by set_clock (lives as long as the context)
@@ -571,6 +572,7 @@ static glbm_status finish_create(glbm_ctx *c, const glbm_config *cfgs, int n, vo
     if (!c->buf[0] || !c->buf[1] || !c->d_ip || !c->d_status || !c->d_mom || !c->d_mw || !c->d_part ||
         !c->d_sums)
         return fail(GLBM_E_NOMEM, "device allocation of %.1f MB failed", 2.0 * bytes_state(c) / 1e6);
+    if (c->dims == 1) c->run1d = glbm_plan_run1d(c->geo[0].N, c->prec, c->geo[0].Lx, n);
     CUDA_TRY(cudaMemcpyAsync(c->d_ip, c->h_ip.data(), sizeof(InstParams) * n, cudaMemcpyHostToDevice,
                              c->stream));
     CUDA_TRY(cudaMemsetAsync(c->d_status, 0, ST_WORDS * sizeof(unsigned), c->stream));
@@ -1200,20 +1202,37 @@ static glbm_status step_1d_instance(glbm_ctx *c, int i, int64_t n, int64_t *comp
     return GLBM_OK;
 }
 
+// Whether a call of n steps of one instance that one CTA does not hold is too short
+// for the cluster, which loads and stores the whole lattice from 16 SMs: launch after
+// launch is then faster. Call times on GB300 in us, launches against cluster: FP32
+// D1Q7 x 8000 27.7 and 30.5 for one step, 33.5 and 30.5 for two; D1Q3 x 48000 28.2 and
+// 32.6 for one; D1Q17 x 8000 33.4 and 42.7 for two, 43.1 and 44.2 for four; D1Q17 x 2400
+// 36.3 and 30.7 for one. With r = Q L / 256000 the cluster's share of a launch's time
+// per step (glbm_plan_run1d), the launches' n (1 - r) steps are short of what the
+// cluster loads in about 1.4 + 0.6 r of them; from level 4 on a single launch takes 7 us
+// more, as much as a small lattice's load. FP64, one step: D1Q17 x 1500 37.9 and 42.8,
+// D1Q13 x 2500 36.1 and 42.9, D1Q13 x 2400 35.5 and 34.9, D1Q5 x 3000 36.5 and 30.6.
+static bool short_1d(const glbm_ctx *c, int64_t n)
+{
+    const Geo &g = c->geo[0];
+    const double ql = (double)g.Q * g.Lx;
+    if (c->n_inst > 1 || 2 * ql * c->elem <= 200 * 1024) return false;
+    if (c->prec == GLBM_FP64) return n == 1 && (g.N == 8 || (g.N >= 6 && ql >= 32000));
+    const double r = ql / 256000;
+    return n * (1 - r) < 1.4 + 0.6 * r && !(g.N >= 4 && r < 0.4);
+}
+
 // n steps of every 1D instance in one launch of clusters, from the current buffer
-// into the other one. *done is false, and the state unchanged, where the cluster
-// does not hold the lattice or a node left the positivity domain: the instances
-// are then stepped one after another (step_1d_instance), which stops at the
-// failing step.
+// into the other one. *done is false, and the state unchanged, where a node left the
+// positivity domain: the instances are then stepped one after another
+// (step_1d_instance), which stops at the failing step.
 static glbm_status step_1d_clusters(glbm_ctx *c, int64_t n, bool *done)
 {
     *done = false;
     AuxArgs a = aux_args(c, 0);
     a.inst_stride = c->n_inst > 1 ? c->geo[1].off : 0;
-    int ok = 0;
-    CUDA_TRY(glbm_launch_run1d_cluster(a, inst_ptr(c, c->cur, 0), inst_ptr(c, 1 - c->cur, 0), c->n_inst,
-                                       n, c->d_status, c->stream, &ok));
-    if (!ok) return GLBM_OK;
+    CUDA_TRY(glbm_launch_run1d_cluster(c->run1d, a, inst_ptr(c, c->cur, 0), inst_ptr(c, 1 - c->cur, 0),
+                                       c->n_inst, n, c->d_status, c->stream));
     c->launches += 1;
     glbm_status st = read_status(c);
     if (st != GLBM_OK) return st;
@@ -1307,7 +1326,7 @@ extern "C" glbm_status glbm_step(glbm_ctx *c, int64_t n)
         // takes its place; without memory for it the instances step one after another)
         const int64_t most = (int64_t)1 << 16;
         const bool keep = c->n_inst > 1 && n > most;
-        bool run = n > 0 && !c->halted;
+        bool run = n > 0 && !c->halted && c->run1d.C > 0 && !short_1d(c, n);
         if (run && keep) {
             const glbm_status st = spare_ready(c);
             if (st != GLBM_OK && st != GLBM_E_NOMEM) return st;

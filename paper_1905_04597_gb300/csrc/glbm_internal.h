@@ -358,10 +358,15 @@ int glbm_field_sum_blocks(long long n);
 cudaError_t glbm_launch_step1d(const AuxArgs &a, const void *fin, void *fout, int inst,
                                unsigned *status, cudaStream_t s);
 // `steps` steps of n_inst 1D lattices (instances a.inst_stride elements apart) from f
-// into out, each on a cluster of CTAs (glbm_run1d.cu). *ok is 0, and nothing was
-// launched, for lattices the cluster does not hold.
-cudaError_t glbm_launch_run1d_cluster(const AuxArgs &a, const void *f, void *out, int n_inst,
-                                      long long steps, unsigned *status, cudaStream_t s, int *ok);
+// into out, each on a cluster of CTAs (glbm_run1d.cu), after a plan made once for
+// the context's lattices; C = 0: not on a cluster.
+struct Run1DPlan {
+    int C, m, maxn, threads;  // CTAs per lattice, steps per exchange, largest chunk
+    size_t smem;
+};
+Run1DPlan glbm_plan_run1d(int N, int prec, int L, int n_inst);
+cudaError_t glbm_launch_run1d_cluster(const Run1DPlan &p, const AuxArgs &a, const void *f, void *out,
+                                      int n_inst, long long steps, unsigned *status, cudaStream_t s);
 cudaError_t glbm_launch_run1d_resident(const AuxArgs &a, void *f, int inst, long long steps,
                                        unsigned *status, cudaStream_t s, int *ok);
 

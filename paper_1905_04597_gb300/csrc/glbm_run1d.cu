@@ -180,90 +180,128 @@ __global__ void __launch_bounds__(RUN1D_THREADS) k_run1d_cluster(const __grid_co
     if (bad) flag_unstable(r.status);
 }
 
+void fill_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[1], int C, int ctas, int threads,
+                 size_t smem, cudaStream_t s)
+{
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+}
+
+// The plan of a kernel: chunks, steps per exchange and the launch's shape. C stays 0
+// for lattices that a cluster does not hold.
 template <int N, typename T>
-cudaError_t launch_n(Run1DArgs &r, int n_inst, cudaStream_t s, int *ok)
+void plan_n(int L, Run1DPlan &p)
 {
     constexpr int Q1 = 2 * N + 1;
     auto *const kern = k_run1d_cluster<N, T>;
-    const int L = r.a.Lx;
     // chunks of at least 32 nodes; clusters of 16 CTAs are opt-in
     int C = 16;
     while (C > 1 && L / C < 32) C /= 2;
-    for (;; C /= 2) {
-        r.C = C;
-        r.maxn = (L + C - 1) / C;
+    for (; C >= 1; C /= 2) {
+        const int maxn = (L + C - 1) / C;
         // steps per exchange: as many as 16, with the halos inside four warps (one
         // per SM sub-partition) or one more warp than the chunk has, and within the
         // neighbour's chunk
-        const int warps = r.maxn / 32 + 1 > 4 ? r.maxn / 32 + 1 : 4;
-        int m = (32 * warps - r.maxn) / (2 * N);
+        const int warps = maxn / 32 + 1 > 4 ? maxn / 32 + 1 : 4;
+        int m = (32 * warps - maxn) / (2 * N);
         m = m > 16 ? 16 : m;
         if (m > L / C / N) m = L / C / N;
-        r.m = m < 1 ? 1 : m;
-        const int H = N * r.m;
-        if (H > L / C) return cudaSuccess;  // shorter than the reach: the caller's other paths
-        const size_t smem = sizeof(T) * Q1 * (2 * (size_t)(r.maxn + 2 * H) + 4 * (size_t)H);
-        if (smem > RUN1D_SMEM) return cudaSuccess;
-        // (one limit for every launch: a smaller one set by another thread in between
-        // would refuse this one)
+        m = m < 1 ? 1 : m;
+        const int H = N * m;
+        if (H > L / C) return;  // shorter than the reach: the caller's other paths
+        const size_t smem = sizeof(T) * Q1 * (2 * (size_t)(maxn + 2 * H) + 4 * (size_t)H);
+        if (smem > RUN1D_SMEM) return;
+        // (one limit for every plan: the kernel is shared by contexts of other sizes)
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RUN1D_SMEM);
         if (e == cudaSuccess && C > 8)
             e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-        int threads = (r.maxn + 2 * H + 31) / 32 * 32;
+        int threads = (maxn + 2 * H + 31) / 32 * 32;
         threads = threads > RUN1D_THREADS ? RUN1D_THREADS : threads;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(C * n_inst);
-        cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = s;
         cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = C;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        fill_config(cfg, attr, C, C, threads, smem, nullptr);
         int clusters = 0;
-        e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
-        if (e != cudaSuccess || clusters < 1) {
-            cudaGetLastError();
-            if (C > 8) continue;  // no GPC holds 16 CTAs: the portable size
-            return cudaSuccess;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
+        if (e == cudaSuccess && clusters >= 1) {
+            p.C = C;
+            p.m = m;
+            p.maxn = maxn;
+            p.threads = threads;
+            p.smem = smem;
+            return;
         }
-        e = cudaLaunchKernelEx(&cfg, kern, r);
-        if (e == cudaSuccess) *ok = 1;
-        return e;
+        cudaGetLastError();
+        if (C <= 8) return;  // (no GPC holds 16 CTAs: the portable size)
     }
 }
 
-template <typename T>
-cudaError_t launch_t(Run1DArgs &r, int n_inst, cudaStream_t s, int *ok)
+template <int N, typename T>
+cudaError_t launch_n(const Run1DPlan &p, const Run1DArgs &r, int n_inst, cudaStream_t s)
 {
-    switch (r.a.N) {
-#define GLBM_CASE(NN) \
-    case NN: return launch_n<NN, T>(r, n_inst, s, ok);
-        GLBM_CASE(1) GLBM_CASE(2) GLBM_CASE(3) GLBM_CASE(4)
-        GLBM_CASE(5) GLBM_CASE(6) GLBM_CASE(7) GLBM_CASE(8)
-#undef GLBM_CASE
-    default: return cudaErrorInvalidValue;
-    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    fill_config(cfg, attr, p.C, p.C * n_inst, p.threads, p.smem, s);
+    return cudaLaunchKernelEx(&cfg, k_run1d_cluster<N, T>, r);
 }
 
 }  // namespace
 
-cudaError_t glbm_launch_run1d_cluster(const AuxArgs &a, const void *f, void *out, int n_inst,
-                                      long long steps, unsigned *status, cudaStream_t s, int *ok)
+#define GLBM_LEVELS_1D GLBM_CASE(1) GLBM_CASE(2) GLBM_CASE(3) GLBM_CASE(4) \
+                       GLBM_CASE(5) GLBM_CASE(6) GLBM_CASE(7) GLBM_CASE(8)
+
+Run1DPlan glbm_plan_run1d(int N, int prec, int L, int n_inst)
 {
-    *ok = 0;
-    // beyond 3072 nodes FP64 has more warps per SM than pipes to hide them: one
-    // launch per step over the whole chip is as fast
-    if (a.prec == GLBM_FP64 && a.Lx > 3072) return cudaSuccess;
+    Run1DPlan p = {};
+    const int Q1 = 2 * N + 1;
+    // A cluster has at most 16 of the chip's SMs. In FP64 beyond 3072 nodes it has more
+    // warps per SM than pipes to hide them, and one launch per step over the whole
+    // chip is as fast. One instance alone stops earlier: at D1Q17 from 2900 nodes
+    // (per step, cluster against launches: 2900 13.4 and 14.6 us, 3000 15.5 and 14.5;
+    // D1Q15 12.5 and 12.5 at 3072, D1Q3 to D1Q13 1.07 to 2.5 times as fast there), in
+    // FP32 from Q L = 256000 (D1Q3 64000 4.8 and 6.3 us, 100000 7.4 and 6.3; D1Q5
+    // 50000 6.1 and 6.3, 70000 7.8 and 6.3; D1Q11 24000 6.1 and 6.3, 30000 7.5 and
+    // 6.3; D1Q17 15000 6.0 and 6.3, 17000 7.6 and 6.3). Several instances run side by
+    // side in clusters but one after another in launches (two: 1.6 times as fast at
+    // those sizes). Measured on GB300 in calls of 200 steps.
+    if (prec == GLBM_FP64 && L > (N == 8 && n_inst == 1 ? 2900 : 3072)) return p;
+    if (prec != GLBM_FP64 && n_inst == 1 && (long long)Q1 * L > 256000) return p;
+    switch (N) {
+#define GLBM_CASE(NN) \
+    case NN: prec == GLBM_FP64 ? plan_n<NN, double>(L, p) : plan_n<NN, float>(L, p); break;
+        GLBM_LEVELS_1D
+#undef GLBM_CASE
+    default: break;
+    }
+    return p;
+}
+
+cudaError_t glbm_launch_run1d_cluster(const Run1DPlan &p, const AuxArgs &a, const void *f, void *out,
+                                      int n_inst, long long steps, unsigned *status, cudaStream_t s)
+{
     Run1DArgs r;
     r.a = a;
     r.f = f;
     r.out = out;
     r.steps = steps;
     r.status = status;
-    return a.prec == GLBM_FP64 ? launch_t<double>(r, n_inst, s, ok) : launch_t<float>(r, n_inst, s, ok);
+    r.C = p.C;
+    r.m = p.m;
+    r.maxn = p.maxn;
+    switch (a.N) {
+#define GLBM_CASE(NN)                                                   \
+    case NN:                                                            \
+        return a.prec == GLBM_FP64 ? launch_n<NN, double>(p, r, n_inst, s) \
+                                   : launch_n<NN, float>(p, r, n_inst, s);
+        GLBM_LEVELS_1D
+#undef GLBM_CASE
+    default: return cudaErrorInvalidValue;
+    }
 }
