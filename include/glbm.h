@@ -447,12 +447,15 @@ glbm_status glbm_autotune(glbm_ctx *ctx, int reps, double *us);
  * per column and wall into a small device buffer (mode 1, one more launch per
  * step). The sums are the same, in the same order: both modes give identical
  * results. A new context takes mode 1 where the tiles near the walls would
- * repeat the sums for more than a tenth of a step's own loads (in FP32 up to k = 7,
- * whose steps then take dataflow chunks, more than a fifth: high levels,
- * narrow channels), else mode 0. glbm_set_wall_launch sets the mode (0 or 1;
+ * repeat the sums for more than a tenth of a step's own loads (high levels,
+ * narrow channels), else mode 0. In FP32 up to k = 7, where that share lies between
+ * a tenth and a fifth, the measured speed decides by the kind of lattice, the level
+ * and the size: dataflow chunks with the sums in the tiles or steps launched one
+ * after another, and for those either mode. glbm_set_wall_launch sets the mode (0 or 1;
  * -1 restores that default; GLBM_E_INVAL otherwise, GLBM_E_UNSUPPORTED for a
  * context without walls, a batch of mixed levels or a 3D context;
- * synchronises). glbm_get_wall_launch returns the mode, -1 where none applies.
+ * synchronises). glbm_get_wall_launch returns the mode of the steps as glbm_step
+ * takes them, -1 where none applies.
  */
 glbm_status glbm_set_wall_launch(glbm_ctx *ctx, int mode);
 int glbm_get_wall_launch(const glbm_ctx *ctx);

@@ -105,6 +105,12 @@ struct ChunkGraph {
     cudaGraphExec_t exec;
 };
 
+// Which steps compute their wall densities in a launch of their own: all, or those
+// outside of dataflow chunks, and whether there are dataflow chunks.
+struct WallMode {
+    bool launch, single, df;
+};
+
 struct glbm_ctx {
     int n_inst = 0;
     int dims = 2, prec = 0;
@@ -135,7 +141,8 @@ struct glbm_ctx {
     double *d_stage = nullptr;     // staging of host inputs
     size_t stage_len = 0;
     void *d_rw = nullptr;          // wall densities of the current step (k_wall_rho)
-    bool wall_launch = false;      // whether k_wall_rho computes them (else each wall tile)
+    WallMode wall = {false, false, true};  // which steps k_wall_rho computes them for (else each
+                                           // wall tile), and whether those allow dataflow chunks
     int4 *d_items = nullptr;       // heterogeneous work list, sorted by level
     int n_items = 0;
     int group[GLBM_MAXN + 2] = {0};  // first item of each level
@@ -476,10 +483,6 @@ static glbm_status ensure_stage(glbm_ctx *c, size_t n)
 // once per column and wall) instead of the prologue of every tile within reach
 // of a wall: when those tiles, at one node row each, would repeat the wall sums
 // for more than 1/share of the step's own loads. Uniform 2D lattices with walls.
-// The share is a tenth, and a fifth in FP32 up to level 8, where a step without
-// that launch takes dataflow chunks (GB300, us per step, own launch against tiles
-// with dataflow: D1Q3 x D1Q8 1000 x 200 x 3 at 14 % 26.6 and 22.2, D2Q121 256 x 128
-// at 11 % 10.1 and 9.2, D2Q289 1024 x 128 x 8 at 26 % 476 and 591).
 static bool wall_rho_pays(int N, int NX, int zv, int Ly, int share)
 {
     const bool zy = (zv & GLBM_ZV_Y) != 0, zx = (zv & GLBM_ZV_X) != 0;
@@ -496,11 +499,51 @@ static bool wall_rho_possible(const glbm_ctx *c)
 {
     return c->dims == 2 && !c->hetero && c->cfg[0].bc == GLBM_BC_WALLS;
 }
-static bool wall_rho_launch(const glbm_ctx *c)
+// The default: the launch above a share of a tenth. In FP32 up to level 8 the overlap of
+// dataflow chunks can hide the repeated sums of a share between a tenth and a fifth. On
+// small lattices it does not (the wall tiles of every step wait for those of the step
+// before: a chain with the sums in it), nor far beyond the L2, where the loads
+// count; and steps that are launched one after another (dataflow off, calls of one
+// step, the adjoint's recomputed steps) are faster without a second launch where they
+// are short. Per kind of lattice and level, in millions of populations of a step: the
+// range lo..hi in which dataflow chunks with the sums in the tiles are the default,
+// and the size from which other steps take the launch. GB300, us per step, launch /
+// dataflow / tiles one after another: D2Q49 1000 x 48 x 2 11.4 / 7.4 / 10.4; D2Q81
+// 64 x 84 (0.4 M) 6.5 / 7.6 / 6.8, 1000 x 59 x 2 (9.6 M) 16.9 / 13.0 / 17.5; D2Q121
+// 1000 x 90 x 4 (44 M) 68.9 / 71.1 / 72.3; D2Q169 256 x 129 (5.6 M) 14.8 / 10.8 /
+// 15.1, 1000 x 129 x 4 (87 M) 165 / 192 / 176; D1Q3 x D1Q8 1000 x 143 x 4 24.8 / 21.0 /
+// 25.1; D1Q3 x D1Q18 64 x 1020 (3.5 M) 14.4 / 17.4 / 15.7, 256 x 1020 (14 M) 33.8 /
+// 26.6 / 40.8. Above a fifth the launch stays (D2Q289 1024 x 128 x 8 at 26 % 476 / 591).
+struct WallRange {
+    float lo, hi, single;
+};
+static const float kAll = 1e9f;
+static const WallRange kWallRange[5][7] = {
+    // levels 2..8: isotropic
+    {{0, kAll, kAll}, {0, kAll, kAll}, {3.2f, 28, 6}, {1.2f, 32, 13}, {1.7f, 27, 3.5f}, {4.2f, 55, 4}, {2.2f, 33, 6}},
+    // D1Q3 along x
+    {{0, kAll, kAll}, {0, kAll, kAll}, {0, kAll, kAll}, {2, 30, 11}, {3.6f, 29, 5}, {4.1f, 31, 2.5f}, {3.6f, 33, 0}},
+    // D1Q3 along x, 2N+2 along y
+    {{0, kAll, kAll}, {1, 27, kAll}, {2.6f, 30, 5}, {3.1f, 40, 0}, {4.3f, 36, 0}, {4.8f, 45, 0}, {4.7f, 40, 0}},
+    // 2N+2 along both axes
+    {{0, kAll, kAll}, {1.2f, 55, kAll}, {2.3f, 33, 12}, {4, 65, 0}, {5.5f, 95, 0}, {3, 95, 0}, {4, 29, 0}},
+    // isotropic with Guo's force
+    {{0, kAll, kAll}, {0, kAll, kAll}, {0, kAll, kAll}, {1.1f, 12, 11}, {1.6f, 26, 3.5f}, {2, 27, 5.5f}, {1.3f, 22, 3}},
+};
+
+static WallMode wall_default(const glbm_ctx *c)
 {
     const Geo &g = c->geo[0];
-    const int share = c->prec == GLBM_FP32_DEV && g.N <= GLBM_MAXN_2N1 ? 5 : 10;
-    return wall_rho_possible(c) && wall_rho_pays(g.N, g.NX, g.zv, g.Ly, share);
+    if (!wall_rho_possible(c) || !wall_rho_pays(g.N, g.NX, g.zv, g.Ly, 10))
+        return WallMode{false, false, true};
+    if (c->prec != GLBM_FP32_DEV || g.N > GLBM_MAXN_2N1 || wall_rho_pays(g.N, g.NX, g.zv, g.Ly, 5))
+        return WallMode{true, false, true};
+    if (g.N < 2) return WallMode{false, false, true};
+    const bool guo = c->cfg[0].force == GLBM_FORCE_GUO;
+    const int kind = g.zv == GLBM_ZV_Y ? 2 : g.zv ? 3 : g.NX != g.N ? 1 : guo ? 4 : 0;
+    const WallRange &w = kWallRange[kind][g.N - 2];
+    const double m = 1e-6 * (double)(c->n_inst * g.Q * g.nodes());
+    return WallMode{false, m >= w.single, m >= w.lo && m <= w.hi};
 }
 static glbm_status alloc_wall_rho(glbm_ctx *c)
 {
@@ -564,10 +607,10 @@ static glbm_status finish_create(glbm_ctx *c, const glbm_config *cfgs, int n, vo
     c->d_mw = (double *)dev_alloc(c->A, 2 * (size_t)max_cols * sizeof(double), c->stream);
     c->d_part = (double *)dev_alloc(c->A, 3 * (size_t)blocks * sizeof(double), c->stream);
     c->d_sums = (double *)dev_alloc(c->A, 3 * sizeof(double), c->stream);
-    if (wall_rho_launch(c)) {
+    c->wall = wall_default(c);
+    if (c->wall.launch || c->wall.single) {
         glbm_status ws = alloc_wall_rho(c);
         if (ws != GLBM_OK) return ws;
-        c->wall_launch = true;
     }
     if (!c->buf[0] || !c->buf[1] || !c->d_ip || !c->d_status || !c->d_mom || !c->d_mw || !c->d_part ||
         !c->d_sums)
@@ -924,10 +967,16 @@ extern "C" size_t glbm_elem_size(const glbm_ctx *c) { return c ? c->elem : 0; }
 // ---------------------------------------------------------------------------
 // stepping
 // ---------------------------------------------------------------------------
-// Arguments of the uniform step from fin into fout; TY is AxisTable for levels
-// up to 8 and AxisTableHi above.
+// Whether k_wall_rho runs before each step (df: of a dataflow chunk).
+static bool wall_steps(const glbm_ctx *c, bool df)
+{
+    return c->wall.launch || (c->wall.single && !df);
+}
+
+// Arguments of the uniform step from fin into fout (df: a step of a dataflow chunk);
+// TY is AxisTable for levels up to 8 and AxisTableHi above.
 template <class TY>
-static Step2DArgsT<TY> step_args_t(const glbm_ctx *c, const void *fin, void *fout)
+static Step2DArgsT<TY> step_args_t(const glbm_ctx *c, const void *fin, void *fout, bool df = false)
 {
     const Geo &g = c->geo[0];
     Step2DArgsT<TY> a;
@@ -943,7 +992,7 @@ static Step2DArgsT<TY> step_args_t(const glbm_ctx *c, const void *fin, void *fou
     a.status = c->d_status;
     a.step_ctr = c->d_status + ST_CLOCK;
     a.done_ctr = c->d_status + ST_DONE;
-    a.rw = c->wall_launch ? c->d_rw : nullptr;
+    a.rw = wall_steps(c, df) ? c->d_rw : nullptr;
     a.Lx = g.Lx;
     a.Ly = g.Ly;
     a.pitch = g.pitch;
@@ -1021,10 +1070,10 @@ static cudaError_t launch_small(const glbm_ctx *c, const void *fin, void *fout, 
 }
 
 // Kernel launches of one 2D step.
-static int launches_per_step(const glbm_ctx *c)
+static int launches_per_step(const glbm_ctx *c, bool df = false)
 {
     if (c->small) return 1;
-    return c->hetero ? glbm_batched_launches(batch_args(c, 0)) : (c->wall_launch ? 2 : 1);
+    return c->hetero ? glbm_batched_launches(batch_args(c, 0)) : (wall_steps(c, df) ? 2 : 1);
 }
 
 // Dataflow chunks (glbm_internal.h): uniform 2D contexts of levels up to 8
@@ -1033,7 +1082,7 @@ static int launches_per_step(const glbm_ctx *c)
 static bool df_eligible(const glbm_ctx *c)
 {
     return c->dataflow && !c->hetero && c->dims == 2 && c->geo[0].N <= GLBM_MAXN_2N1 &&
-           !c->wall_launch && !c->small;
+           !c->wall.launch && c->wall.df && !c->small;
 }
 
 // One 2D (or 3D) step of every instance from state buffer fin into fout, on
@@ -1049,7 +1098,7 @@ static cudaError_t launch_step(const glbm_ctx *c, const void *fin, void *fout, c
     if (N > GLBM_MAXN_2N1)
         return glbm_launch_step2d_zv_hi(N, c->prec, c->tile[N],
                                         step_args_t<AxisTableHi>(c, fin, fout), c->n_inst, s);
-    Step2DArgs a = step_args_t<AxisTable>(c, fin, fout);
+    Step2DArgs a = step_args_t<AxisTable>(c, fin, fout, node >= 0);
     if (node >= 0) {
         a.node_done = c->d_df;
         a.bands = c->d_df + GLBM_DF_CHUNK;
@@ -1149,7 +1198,7 @@ static glbm_status enqueue_steps(glbm_ctx *c, int64_t n, const void *p0, void *p
         } else {
             CUDA_TRY(launch_chunk(c, p0, pa, pb, m, c->stream, df));
         }
-        c->launches += (int64_t)m * launches_per_step(c) + (df ? 1 : 0);  // + k_df_start
+        c->launches += (int64_t)m * launches_per_step(c, df) + (df ? 1 : 0);  // + k_df_start
         void *now = (m & 1) ? pa : pb, *other = (m & 1) ? pb : pa;
         p0 = now;  // the next chunk continues the alternation
         pa = other;
@@ -1859,9 +1908,10 @@ extern "C" glbm_status glbm_set_dataflow(glbm_ctx *c, int on)
 {
     if (!c) return fail(GLBM_E_INVAL, "null context");
     if (on < 0 || on > 2) return fail(GLBM_E_INVAL, "dataflow mode %d (0, 1 or 2)", on);
-    const bool changed = on != c->dataflow || c->small;
+    const bool changed = on != c->dataflow || c->small || !c->wall.df;
     c->dataflow = on;
     c->small = false;
+    c->wall.df = true;  // (as chosen here from now on)
     return changed ? tiles_changed(c) : GLBM_OK;  // the chunk graphs carry the mode
 }
 
@@ -1876,12 +1926,12 @@ extern "C" glbm_status glbm_set_wall_launch(glbm_ctx *c, int mode)
     if (mode < -1 || mode > 1) return fail(GLBM_E_INVAL, "wall launch mode %d (-1, 0 or 1)", mode);
     if (!wall_rho_possible(c))
         return fail(GLBM_E_UNSUPPORTED, "wall densities apply to uniform 2D contexts with walls");
-    const bool on = mode < 0 ? wall_rho_launch(c) : mode == 1;
-    if (on) {
+    const WallMode w = mode < 0 ? wall_default(c) : WallMode{mode == 1, false, true};
+    if (w.launch || w.single) {
         glbm_status st = alloc_wall_rho(c);
         if (st != GLBM_OK) return st;
     }
-    c->wall_launch = on;
+    c->wall = w;
     if (mode >= 0) c->small = false;
     return tiles_changed(c);  // the captured step graphs name the old launches
 }
@@ -1889,7 +1939,7 @@ extern "C" glbm_status glbm_set_wall_launch(glbm_ctx *c, int mode)
 extern "C" int glbm_get_wall_launch(const glbm_ctx *c)
 {
     if (!c || !wall_rho_possible(c)) return -1;
-    return c->wall_launch ? 1 : 0;
+    return wall_steps(c, df_eligible(c)) ? 1 : 0;
 }
 
 extern "C" glbm_status glbm_set_tiles(glbm_ctx *c, const int *tiles)
@@ -1965,7 +2015,7 @@ static glbm_status autotune_dataflow(glbm_ctx *c, cudaEvent_t e0, cudaEvent_t e1
     if (st != GLBM_OK) return st;
     const int64_t steps = 2 * kGraphChunk;
     const int tile0 = c->tile[N];
-    const bool wall0 = c->wall_launch;
+    const bool wall0 = c->wall.launch;
     float best = 0.f;
     st = tiles_changed(c);
     if (st == GLBM_OK) st = time_steps(c, steps, false, e0, e1, &best);
@@ -1975,7 +2025,7 @@ static glbm_status autotune_dataflow(glbm_ctx *c, cudaEvent_t e0, cudaEvent_t e1
     const int n = ctx_tile_shapes(c, N, sh);
     for (int idx = 0; idx < n && st == GLBM_OK; ++idx) {
         c->tile[N] = idx;
-        c->wall_launch = false;
+        c->wall.launch = false;
         st = tiles_changed(c);
         float ms = 0.f;
         if (st == GLBM_OK) st = time_steps(c, steps, true, e0, e1, &ms);
@@ -1987,7 +2037,7 @@ static glbm_status autotune_dataflow(glbm_ctx *c, cudaEvent_t e0, cudaEvent_t e1
         }
     }
     c->tile[N] = best_tile;
-    c->wall_launch = best_wall;
+    c->wall.launch = best_wall;
     c->dataflow = best_df ? 1 : 0;
     return st;
 }
@@ -2014,6 +2064,7 @@ extern "C" glbm_status glbm_autotune(glbm_ctx *c, int reps, double *us)
     glbm_status st = ce == cudaSuccess ? GLBM_OK : fail(GLBM_E_CUDA, "event: %s", cudaGetErrorString(ce));
     const bool small0 = c->small;  // timed against the tuned tiles at the end
     c->small = false;
+    c->wall = WallMode{c->wall.launch, false, true};  // the wall modes are timed one by one
     for (int N = 1; N <= GLBM_MAXN && st == GLBM_OK; ++N) {
         if (!level_present(c, N)) continue;
         TileShape sh[GLBM_MAX_TILES];
@@ -2049,7 +2100,7 @@ extern "C" glbm_status glbm_autotune(glbm_ctx *c, int reps, double *us)
         const int N = c->geo[0].N;
         float ms_mode[2] = {0.f, 0.f};
         for (int m = 0; m < 2 && st == GLBM_OK; ++m) {
-            c->wall_launch = m == 1;
+            c->wall.launch = m == 1;
             cudaError_t e = launch_level_once(c, N);  // warm-up
             if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
             for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch_level_once(c, N);
@@ -2058,7 +2109,7 @@ extern "C" glbm_status glbm_autotune(glbm_ctx *c, int reps, double *us)
             if (e == cudaSuccess) e = cudaEventElapsedTime(&ms_mode[m], e0, e1);
             if (e != cudaSuccess) st = fail(GLBM_E_CUDA, "autotune launch: %s", cudaGetErrorString(e));
         }
-        c->wall_launch = ms_mode[1] < ms_mode[0];
+        c->wall.launch = ms_mode[1] < ms_mode[0];
     }
     // and last, for contexts that can step in dataflow chunks, whole chunks of
     // steps both ways (a launch timed alone cannot show the overlap)
