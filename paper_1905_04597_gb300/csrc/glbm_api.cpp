@@ -1040,6 +1040,7 @@ static BatchArgs batch_args(const glbm_ctx *c, const void *fin, void *fout)
     b.n_items = c->n_items;
     for (int N = 0; N <= GLBM_MAXN + 1; ++N) b.group[N] = c->group[N];
     for (int N = 0; N <= GLBM_MAXN; ++N) b.shape[N] = c->tile[N];
+    for (const Geo &g : c->geo) b.pops[g.N] += g.Q * g.nodes();
     b.status = c->d_status;
     b.step_ctr = c->d_status + ST_CLOCK;
     b.done_ctr = c->d_status + ST_DONE;

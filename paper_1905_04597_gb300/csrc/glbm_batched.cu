@@ -1,8 +1,10 @@
 // Launch sequence of one heterogeneous-batch step: one launch per level present,
 // dealt to the context's stream and two side streams (the kernels are in
-// glbm_batched.cuh). One stream left the chip partly idle at the end of each of the
-// up to eight launches of 10 to 85 us (GB300, 64 channels of levels 2..8 and 64 columns,
-// 20 steps with states set and moments read: 8.41 -> 8.16 ms).
+// glbm_batched.cuh). One stream left the chip partly idle at the end of each of the up
+// to eight launches. GB300, us per step, one stream and three: 7 channels of levels 2 to
+// 8 and 64 x 200 nodes 68.7 and 48.3, 21 of them 125 and 111, 63 of 64 x 60 125 and 110,
+// of 16 x 40 88 and 58; 63 of 64 x 200 250 and 250 (in chunks; 279 and 268 in calls of
+// 8 steps); levels 2 to 4, 3 channels of 16 x 40 16.6 and 7.5.
 #include <algorithm>
 
 #include "glbm_internal.h"
@@ -31,16 +33,15 @@ cudaError_t glbm_launch_batched_level(int N, const BatchArgs &a, bool advance, c
 
 cudaError_t glbm_launch_batched_f32(const BatchArgs &a, cudaStream_t s, const SideStreams &side)
 {
-    // the levels in order of decreasing work (items times populations per node), each
-    // to the stream with the least work so far
+    // the levels in order of decreasing work (populations), each to the stream with the
+    // least work so far
     struct Level {
         int N;
         long long work;
     } lv[GLBM_MAXN_2N1];
     int n = 0;
     for (int N = 1; N <= GLBM_MAXN_2N1; ++N) {
-        const long long items = a.group[N + 1] - a.group[N];
-        if (items > 0) lv[n++] = Level{N, items * (2 * N + 1) * (2 * N + 1)};
+        if (a.pops[N] > 0) lv[n++] = Level{N, a.pops[N]};
     }
     std::sort(lv, lv + n, [](const Level &x, const Level &y) { return x.work > y.work; });
     const int used = std::min(n, GLBM_SIDE_STREAMS + 1);

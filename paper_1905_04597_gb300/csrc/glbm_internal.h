@@ -216,6 +216,7 @@ struct BatchArgs {
     int n_items;
     int group[GLBM_MAXN + 2];  // items of level N: [group[N], group[N + 1]) (group[0] unused)
     int shape[GLBM_MAXN + 1];  // FP32 tile shape index of each level
+    long long pops[GLBM_MAXN + 1];  // populations of each level
     unsigned *status, *step_ctr, *done_ctr;
 };
 // The same for one level's launch.
