@@ -395,7 +395,9 @@ glbm_status glbm_adjoint_flowrate(glbm_ctx *ctx, int64_t steps, int64_t ckpt_eve
  * node rows: each thread updates V x-adjacent nodes (V = 2: FP32 pairs with
  * packed two-lane arithmetic), and each node's 2k+3 velocity rows are dealt
  * to G warps. Every level k (0..GLBM_LEVELS-1) and precision has up to
- * GLBM_MAX_TILES candidate shapes; entry 0 is the default of a new context.
+ * GLBM_MAX_TILES candidate shapes; entry 0 is the default of a new context
+ * (glbm_batch_create: at k = 5 and 6 another entry of the same G where it suits the
+ * batch's widths, with the same results; glbm_get_tiles tells).
  * New uniform FP64 contexts of small lattices with the linearised force step with
  * a kernel of their own instead (one thread per node and velocity row, the
  * results those of entry 0 bit for bit; no dataflow chunks and no wall-density

@@ -726,6 +726,26 @@ static TileShape tile_of(const glbm_ctx *c, int N)
     return n > 0 ? sh[c->tile[N] < n ? c->tile[N] : 0] : TileShape{1, 1, 1};
 }
 
+// The tile shapes a batch starts with: entry 0 of each level, but at levels 6 and 7 the
+// entry of the same G (same results) that is faster in batches. Level 7: (5, 1, 1)
+// (batches of 4 and 16 channels of 32 to 1024 columns, 128 rows, GB300: 1.08 to 1.98
+// times as fast as (5, 1, 2)). Level 6: the pair tile (4, 1, 2), where its 64 columns
+// take hardly more padding than 32 do and its CTAs are more than five per SM (us
+// per step against (4, 2, 1), 4 channels: 64 columns, 512 CTAs 17.3 and 15.7, 96 24.9
+// and 20.7, 128 25.7 and 26.7; 16 channels: 32 columns 48.1 and 27.6, 48 50.4 and 55.9,
+// 64 50.3 and 55.5, 96 88.1 and 78.3, 512 320 and 369).
+static void choose_batch_tiles(glbm_ctx *c)
+{
+    long long pairs = 0, singles = 0;  // node rows of 64 and of 32 columns at level 6
+    for (const Geo &g : c->geo) {
+        if (g.N != 6) continue;
+        pairs += (long long)((g.Lx + 63) / 64) * g.Ly;
+        singles += (long long)((g.Lx + 31) / 32) * g.Ly;
+    }
+    c->tile[6] = pairs > 5 * 152 && 50 * pairs <= 27 * singles ? 2 : 0;  // (8 % more)
+    c->tile[7] = 1;
+}
+
 // Work list of a heterogeneous batch: every (instance, tile) with the rows of
 // its level's tile shape, grouped by level (instance order within a level).
 static glbm_status build_items(glbm_ctx *c)
@@ -776,12 +796,8 @@ extern "C" glbm_status glbm_batch_create(const glbm_config *cfgs, int n, void *s
     glbm_ctx *c = new (std::nothrow) glbm_ctx();
     if (!c) return fail(GLBM_E_NOMEM, "host allocation failed");
     c->hetero = true;
-    // batches hold narrow channels: the entry of the default's G (same results) that
-    // was faster there (GB300, 64 channels of 64 columns, us per launch): (4, 1, 2)
-    // 76.4 against (4, 2, 1) 83.8 at N = 6, (5, 1, 1) 46.3 against (5, 1, 2) 49.4 at 7
-    c->tile[6] = 2;
-    c->tile[7] = 1;
     glbm_status st = finish_create(c, cfgs, n, stream);
+    if (st == GLBM_OK) choose_batch_tiles(c);
     if (st == GLBM_OK) st = create_side_streams(c);
     if (st == GLBM_OK) st = build_items(c);
     if (st != GLBM_OK) {
