@@ -238,7 +238,9 @@ glbm_status glbm_sync(glbm_ctx *ctx);
  *   bit 6 sigma_xy = sum (xi_x-u_x)(xi_y-u_y) f.
  * In 1D only bits 0, 1, 3, 4 apply. 3D lattices (fields nz*ny*nx values
  * [z][y][x]) add bit 7 u_z and bit 8 q_z, with T = sum |xi-u|^2 f / (3 rho).
- * `out_len` is the capacity in doubles.
+ * `out_len` is the capacity in doubles. out_on_device: memory that a copy on the
+ * device reaches; the context's own GPU's is written by the kernel, another GPU's and
+ * managed memory by a copy from the context's buffer.
  * Synchronises the stream when out is host memory. */
 #define GLBM_M_RHO 0x01u
 #define GLBM_M_UX 0x02u

@@ -1554,6 +1554,17 @@ extern "C" glbm_status glbm_channel_diagnostics(glbm_ctx *c, int inst, double *p
     return GLBM_OK;
 }
 
+// Whether the kernels of this call may write p.
+static bool on_this_device(const void *p)
+{
+    cudaPointerAttributes a = {};
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaPointerGetAttributes(&a, p);
+    if (e != cudaSuccess) cudaGetLastError();
+    return glbm_kernel_may_write(e, a, dev);
+}
+
 extern "C" glbm_status glbm_moments(glbm_ctx *c, int inst, unsigned mask, double *out,
                                     size_t out_len, int out_on_device)
 {
@@ -1574,12 +1585,14 @@ extern "C" glbm_status glbm_moments(glbm_ctx *c, int inst, unsigned mask, double
     }
     if (need == 0) return fail(GLBM_E_INVAL, "empty field mask");
     if (out_len < need) return fail(GLBM_E_INVAL, "output holds %zu doubles, needs %zu", out_len, need);
-    st = compute_moments(c, inst, mask, out_on_device ? out : c->d_mom);
+    const bool direct = out_on_device && on_this_device(out);
+    st = compute_moments(c, inst, mask, direct ? out : c->d_mom);
     if (st != GLBM_OK) return st;
-    if (!out_on_device) {
-        CUDA_TRY(cudaMemcpyAsync(out, c->d_mom, need * 8, cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(cudaStreamSynchronize(c->stream));
-    }
+    if (!direct)
+        CUDA_TRY(cudaMemcpyAsync(out, c->d_mom, need * 8,
+                                 out_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                                 c->stream));
+    if (!out_on_device) CUDA_TRY(cudaStreamSynchronize(c->stream));
     return GLBM_OK;
 }
 

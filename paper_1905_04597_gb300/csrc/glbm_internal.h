@@ -331,6 +331,13 @@ cudaError_t glbm_launch_set_populations(const AuxArgs &a, void *f, const double 
                                         unsigned *status, cudaStream_t s);
 cudaError_t glbm_launch_get_populations(const AuxArgs &a, const void *f, double *dst,
                                         cudaStream_t s);
+// Whether a kernel on device `dev` may write the memory that cudaPointerGetAttributes
+// described with status e: that device's own. Other memory that a copy reaches (another
+// GPU's, managed or pinned host memory) is copied to.
+inline bool glbm_kernel_may_write(cudaError_t e, const cudaPointerAttributes &a, int dev)
+{
+    return e == cudaSuccess && a.type == cudaMemoryTypeDevice && a.device == dev;
+}
 // Destinations of the moment fields, by the bit of GLBM_M_*; null: not wanted.
 struct MomPtrs {
     double *p[9];
