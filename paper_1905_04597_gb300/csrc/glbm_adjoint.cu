@@ -34,7 +34,8 @@
 // node, and forms every contraction from row sums: with d = E - W per axis,
 //   sum_i lambda E^x   = sum lambda d^x + sum lambda W^x   (per row),
 //   lambda . (f^eq - f) = rho E^y sum lambda d^x + B sum lambda W^x - sum lambda delta,
-//   B = rho E^y - W^y, delta = f - W,
+//   B = rho E^y - W^y, delta = f - W (FP64 states, which may have any density: with
+//   rho W^y and rho W in place of W^y and W),
 // five FP64 instructions per population for all contractions and two for mu_t, no
 // term larger than the deviations. The wall sums of mu and the wall densities of
 // X_t have a launch of their own (once per column, spread over the chip). D2Q121
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(32 * ADJ_G<N>, ADJ_CTAS<N>)
     using ACC = std::conditional_t<DEV, MomAccI<2, N, 0, false>, MomAccD<2, N, 0, false>>;
     __shared__ double eq[4][Q1][32];   // d^x, dE^x, d^y, dE^y
     __shared__ double con[G][5][32];   // the groups' partial moments, then contractions
-    __shared__ double rup[3][32];      // rho - 1, u_x, u_y
+    __shared__ double rup[3][32];      // rho (FP32 states: rho - 1), u_x, u_y
     __shared__ double tot[5][32];      // the contractions' totals
     wait_prior_grid();
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
@@ -267,12 +268,13 @@ __global__ void __launch_bounds__(32 * ADJ_G<N>, ADJ_CTAS<N>)
             for (int k = 0; k < 3; ++k) m[k] += con[t][k][lane];
         }
         const double rho = DEV ? 1.0 + m[0] : m[0], inv = 1.0 / rho;
-        rup[0][lane] = DEV ? m[0] : m[0] - 1.0;
+        rup[0][lane] = m[0];
         rup[1][lane] = mom_div(m[1], rho, inv);
         rup[2][lane] = mom_div(m[2], rho, inv);
     }
     __syncthreads();
-    const double drho = rup[0][lane], rho = 1.0 + drho, ux = rup[1][lane], uy = rup[2][lane];
+    const double dens = rup[0][lane], rho = DEV ? 1.0 + dens : dens;
+    const double ux = rup[1][lane], uy = rup[2][lane];
     // the equilibrium and its slopes: group g evaluates the (|n|, axis) pairs g,
     // g + G, ...
 #pragma unroll
@@ -296,7 +298,7 @@ __global__ void __launch_bounds__(32 * ADJ_G<N>, ADJ_CTAS<N>)
         const int iy = g + k * G;
         if (iy < Q1) {
             double Ld = 0.0, Lw = 0.0, Ls = 0.0, Lg = 0.0, Lf = 0.0;
-            const double wy = a.tab.W[iy];
+            const double wy = a.tab.W[iy], base = DEV ? wy : rho * wy;
             const int ys = y - (iy - N);
             const bool ghost = walls && (ys < 0 || ys >= a.Ly);
 #pragma unroll
@@ -311,20 +313,22 @@ __global__ void __launch_bounds__(32 * ADJ_G<N>, ADJ_CTAS<N>)
                 const double *const ew = ys < 0 ? ip.ew_lo : ip.ew_hi;
 #pragma unroll
                 for (int ix = 0; ix < Q1; ++ix) Lf = fma(lam[k][ix], ew[ix], Lf);
-                Lf = wy * fma(ys < 0 ? rw_lo : rw_hi, Lf, -Lw);
+                const double rw = ys < 0 ? rw_lo : rw_hi;
+                Lf = DEV ? wy * fma(rw, Lf, -Lw) : fma(wy * rw, Lf, -(base * Lw));
             } else {
 #pragma unroll
                 for (int ix = 0; ix < Q1; ++ix) {
-                    const double d = DEV ? to_f64(f[k][ix]) : fma(-wy, a.tab.W[ix], to_f64(f[k][ix]));
+                    const double d = DEV ? to_f64(f[k][ix]) : fma(-base, a.tab.W[ix], to_f64(f[k][ix]));
                     Lf = fma(lam[k][ix], d, Lf);
                 }
             }
             const double dy = eq[2][iy][lane], L0 = Ld + Lw;
-            const double Ey = wy + dy, B = fma(drho, wy, rho * dy);
+            const double Ey = wy + dy;
+            const double B = DEV ? fma(dens, wy, rho * dy) : fma(rho, dy, fma(rho, wy, -base));
             a0 = fma(Ey, L0, a0);
             ax = fma(Ey, Ls, ax);
             ay = fma(eq[3][iy][lane], L0, ay);
-            gt += fma(wy + B, Ld, fma(B, Lw, -Lf));
+            gt += fma(base + B, Ld, fma(B, Lw, -Lf));
             gg = fma(wy, Lg, gg);
         }
     }
