@@ -10,17 +10,21 @@
 // What bounds it: FP64 needs two instructions and a conversion per population on a
 // pipe that issues two per cycle and SM, fourteen times the time of the stores. FP32
 // deviations are formed in float pairs (value = h + l, 48 bits) on the FP32 pipe
-// instead: the value before the rounding to float is exact to 2^-43 of its terms, and
-// where the rounding could go either way within 2^-41 (about one population in 2^16)
-// it is formed in FP64, so every stored float is that of the FP64 formula. Fields
-// outside 1e-18..1e18 in magnitude (or not finite) take FP64. The pairs' kernel is
-// bound by its issue slots (92 instructions per population at D3Q125 and 65 at D2Q289
-// with run-time row lengths), so the x axis's velocities are a template parameter,
-// populations too close to call are collected and formed after their row, and E^y,
-// rho E^z and rho (E^z - W^z) are formed once per node. Measured on GB300, FP32, FP64
-// pipe -> pairs -> this: D2Q81 512 x 256 95 -> 39 -> 33 us, D2Q289 1024 x 128 311 -> 95
-// -> 79 us, D3Q125 250 x 61 x 45 815 -> 257 -> 183 us; D1Q3 x D1Q28 200 nodes (FP64)
-// 25 -> 10 us; large FP64 lattices stay on the FP64 pipe (D2Q81 54 us).
+// instead. The value before the rounding to float is off by at most 2^-44.4 of the
+// magnitudes of its terms (the largest of 2 x 10^8 populations per level and dimension
+// against FP64, levels 1 to 8 and 13, velocities up to 1), the terms of B and of d taken
+// before they cancel. Where the rounding could go either way within 2^-42 of them (one
+// population in 2^14 to 2^15 at velocities of 0.03) it is formed in FP64, so every
+// stored float is that of the FP64 formula. Fields outside 1e-18..1e18 in magnitude (or
+// not finite) take FP64. The pairs' kernel is bound by its issue slots (92 instructions
+// per population at D3Q125 and 65 at D2Q289 with run-time row lengths), so the x axis's
+// velocities are a template parameter, populations too close to call are collected and
+// formed after their row, and E^y, rho E^z and rho (E^z - W^z) are formed once per node.
+// Measured on GB300, FP32, FP64 pipe -> pairs -> this: D2Q81 512 x 256 95 -> 39 -> 34 us,
+// D2Q289 1024 x 128 311 -> 95 -> 84 us, D3Q125 250 x 61 x 45 815 -> 257 -> 194 us (3 to
+// 6 % of it for the terms' magnitudes; tolerances of |W^x B| + |d^x A| alone left one
+// population in 10^8 a float off, one in 10^4 where rows cancel); D1Q3 x D1Q28 200 nodes
+// (FP64) 25 -> 10 us; large FP64 lattices stay on the FP64 pipe (D2Q81 54 us).
 #include "glbm_device.cuh"
 
 namespace {
@@ -78,6 +82,8 @@ struct F32 {
     static __device__ __forceinline__ V neg(V a) { return df_neg(a); }
 };
 
+constexpr float EQ_V = 0x1p-6f;
+
 // Table of one axis in the arithmetic's values: rest weights by velocity index, and
 // the even and odd coefficients of every mirror pair (Ce[m][i], i = 0..N-1 for v^(i+1)).
 // M: the highest level it holds (kernel parameters of 5 KB at 8, 12 KB at 13).
@@ -86,6 +92,7 @@ struct EqAxis {
     int N, zv;
     V W[2 * M + 2];
     V Ce[M + 1][M], Co[M + 1][M];
+    float me[M + 1], mo[M + 1];  // sums of |Ce| v^i and |Co| v^i at v = EQ_V
 };
 struct NoAxis {};
 template <class V, int M>
@@ -103,12 +110,16 @@ struct EqArgs {
     long long plane;
 };
 
-// E - W of the mirror pair m of one axis (plus: the positive velocity).
+// E - W of the mirror pair m of one axis (plus: the positive velocity). Float pairs:
+// also the sum of its terms' magnitudes, which its error is a fraction of, with 2^-80
+// for the words that underflow at tiny velocities (0 at u = 0, where both are exact):
+// from its sums at v = 2^-6 up to there, term by term beyond.
 template <class P, int M>
 __device__ __forceinline__ void eq_pair(const EqAxis<typename P::V, M> &t, int m, typename P::V u,
-                                        typename P::V &plus, typename P::V &minus)
+                                        typename P::V &plus, typename P::V &minus, float &mag)
 {
     using V = typename P::V;
+    constexpr bool F = std::is_same<V, df>::value;
     const int N = t.N;
     const V v = P::mul(u, u);
     V e = t.Ce[m][N - 1], o = t.Co[m][N - 1];
@@ -117,6 +128,17 @@ __device__ __forceinline__ void eq_pair(const EqAxis<typename P::V, M> &t, int m
         o = P::fma_(o, v, t.Co[m][i]);
     }
     e = P::mul(e, v);
+    if constexpr (F) {
+        float me = t.me[m], mo = t.mo[m];
+        if (v.h > EQ_V) {
+            me = mo = 0.f;
+            for (int i = N - 1; i >= 0; --i) {
+                me = fmaf(me, v.h, fabsf(t.Ce[m][i].h));
+                mo = fmaf(mo, v.h, fabsf(t.Co[m][i].h));
+            }
+        }
+        mag = u.h != 0.f ? fmaf(fabsf(u.h), mo, fmaf(me, v.h, 0x1p-80f)) : 0.f;
+    }
     if (m == 0 && !t.zv) {  // the zero velocity
         plus = minus = e;
         return;
@@ -157,15 +179,15 @@ __device__ __noinline__ float eq_exact(const EqArgs<df, M> &a, int n, int iz, in
     return (float)fma(dev(a.x64, a.u[0] ? a.u[0][n] : 0.0, ix), A, mul_rn(a.x64.W[ix], B));
 }
 
-// W^x B + d^x A rounded once to float; false where the rounding is too close to call.
-__device__ __forceinline__ bool eq_dev(df w, df B, df d, df A, float &out)
+// W^x B + d^x A rounded once to float; false where the rounding is too close to call
+// for an error of up to `tol`.
+__device__ __forceinline__ bool eq_dev(df w, df B, df d, df A, float tol, float &out)
 {
     const float p = __fmul_rn(w.h, B.h), q = __fmul_rn(d.h, A.h);
     const float pe = fmaf(w.l, B.h, fmaf(w.h, B.l, fmaf(w.h, B.h, -p)));
     const float qe = fmaf(d.l, A.h, fmaf(d.h, A.l, fmaf(d.h, A.h, -q)));
     const float s = p + q, t = s - p;
     const float e = ((p - (s - t)) + (q - t)) + (pe + qe);
-    const float tol = 0x1p-41f * (fabsf(p) + fabsf(q));
     out = s + (e - tol);
     return out == s + (e + tol);
 }
@@ -181,10 +203,18 @@ __global__ void __launch_bounds__(32 * EQ_WARPS)
     constexpr bool F = std::is_same<V, df>::value;  // float pairs
     __shared__ V in[5][32];                  // u_x, u_y, u_z, rho, rho - 1
     __shared__ V dx[2 * GLBM_MAXN_2N1 + 2][32];  // FP32: E^x - W^x; FP64: E^x
-    __shared__ V dy[2 * M + 2][32], dz[2 * GLBM_MAXN_3D + 1][32];
-    // float pairs: E^y, and (3D) rho E^z and rho (E^z - W^z)
-    __shared__ V ey[F ? 2 * M + 2 : 1][32], pz[F ? 2 * GLBM_MAXN_3D + 1 : 1][32],
-        qz[F ? 2 * GLBM_MAXN_3D + 1 : 1][32];
+    __shared__ V dy[2 * M + 2][32];              // E^y - W^y
+    // float pairs: E^y, the magnitudes of E^x - W^x's terms by mirror pair, and per row
+    // the tolerances of W^x B and d^x A over the x axis's factors (3D: their factors)
+    __shared__ V ey[F ? 2 * M + 2 : 1][32];
+    __shared__ float magx[F ? GLBM_MAXN_2N1 + 1 : 1][32];
+    __shared__ float2 ty[F ? 2 * M + 2 : 1][32];
+    // 3D: E^z - W^z, and for float pairs rho E^z, rho (E^z - W^z) and the tolerances'
+    // factors, in the rows that its levels leave free
+    constexpr int QZ = 2 * GLBM_MAXN_3D + 1;
+    static_assert(2 * M + 2 >= 2 * QZ, "room for the z axis");
+    V(*const dz)[32] = dy + QZ, (*const pz)[32] = ey + QZ, (*const qz)[32] = dx + QZ;
+    float2(*const tz)[32] = ty + QZ;
     if (a.status && blockIdx.x == 0 && threadIdx.x == 0) reset_status(a.status);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int n = blockIdx.x * 32 + lane, nc = n < a.nodes ? n : a.nodes - 1;
@@ -219,11 +249,24 @@ __global__ void __launch_bounds__(32 * EQ_WARPS)
         const int m = ax == 0 ? t : ax == 1 ? t - nx : t - nx - ny;
         const EqAxis<V, M> &tab = ax == 0 ? a.x : a.y;
         V plus, minus;
-        eq_pair<P>(tab, m, in[ax][lane], plus, minus);
+        float mag;
+        eq_pair<P>(tab, m, in[ax][lane], plus, minus, mag);
         const int ip = tab.zv ? tab.N + 1 + m : tab.N + m, im = tab.N - m;
         if (!F && ax == 0) {
             plus = P::add(tab.W[ip], plus);
             minus = P::add(tab.W[im], minus);
+        }
+        if constexpr (F) {
+            const float w = tab.W[ip].h, ar = 0x1p-42f * fabsf(in[3][lane].h);
+            const float ar1 = 0x1p-42f * fabsf(in[4][lane].h);
+            if (ax == 0)
+                magx[m][lane] = mag;
+            else if (ax == 2)
+                tz[im][lane] = tz[ip][lane] = make_float2(ar * (w + mag), ar * mag);
+            else if (a.dims == 2)
+                ty[im][lane] = ty[ip][lane] = make_float2(ar * (w + mag), fmaf(ar1, w, ar * mag));
+            else
+                ty[im][lane] = ty[ip][lane] = make_float2(w + mag, mag);
         }
         if (F && ax == 1) {
             ey[im][lane] = P::add(tab.W[im], minus);
@@ -246,9 +289,13 @@ __global__ void __launch_bounds__(32 * EQ_WARPS)
     const int rows = a.dims == 3 ? Qy * Qy : Qy;
     const V r = in[3][lane], r1 = in[4][lane];
     const bool live = n < a.nodes, pairs = !((bad >> lane) & 1u);
+    // float pairs: the tolerances of A's and B's terms (1D: of rho and rho - 1)
+    float t0 = 0.f, t1 = 0.f;
+    if constexpr (F) t0 = 0x1p-42f * fabsf(r.h), t1 = 0x1p-42f * fabsf(r1.h);
     int iz = 0, iy = w;
     for (int j = w; j < rows; j += EQ_WARPS, iy += EQ_WARPS) {
         V A = r, B = r1;
+        float tA = t0, tB = t1;
         if (a.dims == 3) {
             for (; iy >= Qy; iy -= Qy) ++iz;
             if constexpr (F) {
@@ -256,6 +303,9 @@ __global__ void __launch_bounds__(32 * EQ_WARPS)
                 A = P::mul(z, ey[iy][lane]);
                 B = P::fma_(r1, a.wyz[iz][iy],
                             P::fma_(dy[iy][lane], z, P::mul(a.y.W[iy], qz[iz][lane])));
+                const float2 fy = ty[iy][lane], fz = tz[iz][lane];
+                tA = fz.x * fy.x;
+                tB = fmaf(t1, a.wyz[iz][iy].h, fmaf(fy.y, fz.x, a.y.W[iy].h * fz.y));
             } else {
                 A = P::mul(r, P::mul(P::add(a.y.W[iy], dy[iy][lane]), P::add(a.y.W[iz], dz[iz][lane])));
             }
@@ -263,6 +313,9 @@ __global__ void __launch_bounds__(32 * EQ_WARPS)
             if constexpr (F) {
                 A = P::mul(r, ey[iy][lane]);
                 B = P::fma_(r1, a.y.W[iy], P::mul(r, dy[iy][lane]));
+                const float2 t = ty[iy][lane];
+                tA = t.x;
+                tB = t.y;
             } else {
                 A = P::mul(r, P::add(a.y.W[iy], dy[iy][lane]));
             }
@@ -274,8 +327,10 @@ __global__ void __launch_bounds__(32 * EQ_WARPS)
             unsigned open = 0u;  // columns to form in FP64
 #pragma unroll
             for (int ix = 0; ix < QX; ++ix, out += a.plane) {
+                constexpr int PX = QX / 2, MX = (QX - 1) / 2;  // columns of the pair number 0
+                const float tol = fmaf(a.x.W[ix].h, tB, magx[ix >= PX ? ix - PX : MX - ix][lane] * tA);
                 float v;
-                if (!eq_dev(a.x.W[ix], B, dx[ix][lane], A, v)) open |= 1u << ix;
+                if (!eq_dev(a.x.W[ix], B, dx[ix][lane], A, tol, v)) open |= 1u << ix;
                 *out = v;
             }
             if (!pairs) open = (1u << QX) - 1u;
@@ -312,6 +367,15 @@ void fill_axis(const AxisTableHi &t, EqAxis<V, M> &e)
             e.Ce[m][i] = host_value(t.Ce[m][i + 1], tag);
             e.Co[m][i] = host_value(m == 0 && !t.zv ? 0.0 : t.Co[m][i], tag);
         }
+    for (int m = 0; m <= t.N; ++m) {
+        double se = 0.0, so = 0.0;
+        for (int i = t.N - 1; i >= 0; --i) {
+            se = se * EQ_V + fabs(t.Ce[m][i + 1]);
+            so = so * EQ_V + (m == 0 && !t.zv ? 0.0 : fabs(t.Co[m][i]));
+        }
+        e.me[m] = (float)se;
+        e.mo[m] = (float)so;
+    }
 }
 
 template <class P, int M>
