@@ -1,10 +1,14 @@
 // Launch sequence of one heterogeneous-batch step: one launch per level present,
 // dealt to the context's stream and two side streams (the kernels are in
 // glbm_batched.cuh). One stream left the chip partly idle at the end of each of the up
-// to eight launches. GB300, us per step, one stream and three: 7 channels of levels 2 to
-// 8 and 64 x 200 nodes 68.7 and 48.3, 21 of them 125 and 111, 63 of 64 x 60 125 and 110,
-// of 16 x 40 88 and 58; 63 of 64 x 200 250 and 250 (in chunks; 279 and 268 in calls of
-// 8 steps); levels 2 to 4, 3 channels of 16 x 40 16.6 and 7.5.
+// to eight launches. Three are faster, but two where five or more levels together fill
+// the chip (from 30 million populations a step): with three, the end of every chain
+// meets fewer other CTAs to fill up with. GB300, us per step in calls of 8 steps, three
+// and two (one in chunks of 64 in brackets): levels 2 to 8, 7 channels of 64 x 60 (4 M)
+// 33.8 and 41.8 (50), 7 of 64 x 200 (13 M) 52.9 and 52.9 (69), 21 of 64 x 200 (38 M) 120
+// and 110 (125), 63 (114 M) 261 and 227 (255), 21 of 512 x 128 (197 M) 409 and 373 (408);
+// levels 2 to 4, 3 of 16 x 40 14.2 and 18.1 (17), 27 of 128 x 300 (55 M) 100 and 103 (103);
+// 64 channels of levels 2 to 8, 64 columns and 32 to 512 rows (138 M) 284 and 262.
 #include <algorithm>
 
 #include "glbm_internal.h"
@@ -44,7 +48,9 @@ cudaError_t glbm_launch_batched_f32(const BatchArgs &a, cudaStream_t s, const Si
         if (a.pops[N] > 0) lv[n++] = Level{N, a.pops[N]};
     }
     std::sort(lv, lv + n, [](const Level &x, const Level &y) { return x.work > y.work; });
-    const int used = std::min(n, GLBM_SIDE_STREAMS + 1);
+    long long total = 0;
+    for (int i = 0; i < n; ++i) total += lv[i].work;
+    const int used = std::min(n, n >= 5 && total > 30000000 ? 2 : GLBM_SIDE_STREAMS + 1);
     cudaError_t e = cudaSuccess;
     if (used > 1) e = cudaEventRecord(side.fork, s);
     for (int k = 0; k + 1 < used && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(side.s[k], side.fork, 0);
