@@ -28,16 +28,17 @@
 //
 // What bounds the adjoint step: the FP64 pipe (two instructions per cycle and SM;
 // mu is FP64, and a step's 79 MB at D2Q121 256 x 128 stay in L2). So the kernel
-// keeps a node's lambda and F in registers (one pull of each instead of three and
-// two), deals its velocity rows to G warps, sums the forward moments of FP32
+// pulls a node's lambda and F once (instead of three times and twice), deals its
+// velocity rows to G warps, sums the forward moments of FP32
 // states in integers (glbm_moments.cuh), evaluates each equilibrium slope once per
 // node, and forms every contraction from row sums: with d = E - W per axis,
 //   sum_i lambda E^x   = sum lambda d^x + sum lambda W^x   (per row),
 //   lambda . (f^eq - f) = rho E^y sum lambda d^x + B sum lambda W^x - sum lambda delta,
 //   B = rho E^y - W^y, delta = f - W (FP64 states, which may have any density: with
 //   rho W^y and rho W in place of W^y and W),
-// five FP64 instructions per population for all contractions and two for mu_t, no
-// term larger than the deviations. The wall sums of mu and the wall densities of
+// five FP64 instructions per population for all contractions and two for mu_t (12 in
+// all with the polynomials, slopes and moments, D2Q121), no term larger than the
+// deviations. The wall sums of mu and the wall densities of
 // X_t have a launch of their own (once per column, spread over the chip). D2Q121
 // 256 x 128, FP32 states, GB300, per step: 350 -> 103 us, the wall sums 65 -> 6 us.
 #include "glbm_moments.cuh"
@@ -131,10 +132,19 @@ __global__ void __launch_bounds__(ADJ_WX *ADJ_WS) k_adj_walls(const __grid_const
     }
 }
 
-// Warps a node's velocity rows are dealt to (three rows per warp: lambda and F stay
-// in registers) and CTAs per SM asked for, 15 or 16 warps where 8 left the FP64
-// pipe 61 % busy between the kernel's barriers (D2Q121 256 x 128: 128 us with 8
-// warps, 103 us with 16; two rows per warp or more warps ran no faster).
+// Warps a node's velocity rows are dealt to (three rows per warp) and CTAs per SM asked
+// for, 15 or 16 warps where 8 left the FP64 pipe 61 % busy between the kernel's
+// barriers (D2Q121 256 x 128: 128 us with 8 warps, 103 us with 16; two rows per warp ran
+// no faster). That caps the registers at 128 (168 at level 8), where part of lambda
+// and F spills from level 4 on (bytes stored and loaded per thread, FP32 and FP64
+// states: level 4 136/216 and 232/336, 5 400/648 and 460/756, 6 572/1164 and 860/1288, 7
+// 760/1512 and 1200/1800, 8 608/1300 and 968/1472), but the warps are worth more than
+// the spills cost: us per step of forward and adjoint at 256 x 128 with a CTA per SM
+// less (levels 5 and up: without spills or nearly) / as here / one more, FP32 states:
+// level 3 69 / 67 / 68, 4 101 / 101 / 102, 5 136 / 127 / 128, 6 197 / 179 / 172, 7 256 /
+// 234 / 221, 8 333 / 311 / 305; FP64: 3 109 / 106 / 107, 4 172 / 176 / 178, 5 232 / 229 /
+// 230, 6 330 / 324 / 302, 7 425 / 421 / 395, 8 560 / 575 / 567. Every level is 1.8 to 4.2
+// times as fast as with one thread per node.
 template <int N>
 constexpr int ADJ_G = N == 1 ? 1 : N == 2 ? 2 : N <= 4 ? 3 : N == 5 ? 4 : N <= 7 ? 5 : 6;
 template <int N>

@@ -1,7 +1,7 @@
-// Auxiliary kernels of libglbm: import/export of populations in the FP64 logical layout, the 1D moment reducer (2D and 3D:
-// glbm_moments.cuh), deterministic global sums, and the 1D step (Sec. 5.1 shock
-// tube, halfway bounce-back) both per launch and resident in one CTA for many
-// steps.
+// Auxiliary kernels of libglbm: import/export of populations in the FP64 logical
+// layout, the 1D moment reducer (2D and 3D: glbm_moments.cuh), deterministic global
+// sums, and the 1D step (Sec. 5.1 shock tube, halfway bounce-back) both per launch
+// and resident in one CTA for many steps.
 #include <algorithm>
 #include <mutex>
 
@@ -9,9 +9,8 @@
 
 namespace {
 
-__device__ __forceinline__ double load_full(const AuxArgs &a, const void *f, long long idx, int q)
+__device__ __forceinline__ double load_full(const AuxArgs &a, const void *f, long long idx)
 {
-    (void)q;
     if (a.prec == GLBM_FP64) return static_cast<const double *>(f)[idx];
     return (double)static_cast<const float *>(f)[idx];
 }
@@ -94,7 +93,7 @@ __global__ void k_moments1d(const __grid_constant__ AuxArgs a, const void *f, Mo
             xs = 2 * a.Lx - 1 - xs;
             n = -n;
         }
-        return load_full(a, f, (long long)(N + n) * a.plane + xs, 0);
+        return load_full(a, f, (long long)(N + n) * a.plane + xs);
     };
     double R0 = pulled(0), R1 = 0.0, R2 = 0.0, R3 = 0.0, c = 0.0;
     double w0 = a.tab.W[N], w2 = 0.0;

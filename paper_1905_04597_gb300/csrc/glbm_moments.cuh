@@ -284,8 +284,10 @@ struct MomAccI {
     }
 };
 
-// j / rho from inv = 1 / rho: one correction rounds like the division; the
-// division itself where the correction is not finite.
+// j / rho from inv, the rounded 1 / rho, by one correction with the exact residual
+// (Markstein's scheme: with a correctly rounded reciprocal the result is the
+// division's but for rare operands, with another one, as 3 rho's below, within an ulp);
+// the division itself where the correction is not finite.
 __device__ __forceinline__ double mom_div(double j, double rho, double inv)
 {
     double q = j * inv;
