@@ -466,22 +466,42 @@ struct Step2D {
                 if constexpr (!DEV) {
                     // f^eq - f0 in one fused rounding, then the force term (skipped
                     // without a force), then f0 + omega (f^eq + F/omega - f0): three
-                    // FP64 instructions, two without a force
-                    T d[QX];
+                    // FP64 instructions, two without a force. Rows of 16 populations and
+                    // more take one after the other, shorter ones the row's differences
+                    // first (GB300, 1024 x 128, us per step, row / one by one: D2Q289 554
+                    // and 456, with a force 627 and 535; D2Q256 518 and 443, 583 and 509;
+                    // D2Q225 348 and 370, 395 and 416; D2Q81 113 and 116)
+                    const auto store = [&](int ix, T d) {
+                        op[ix * plane] = fma(om, d, f[k][ix]);
+                    };
+                    const auto force = [&](int ix, T d) {
+                        const int nx = AX::vel(ix);
+                        if constexpr (GUO)
+                            return fma(A::W(tabx, ix), fma(T(nx), grA, T(AX::ck(ix)) * grB), d);
+                        else
+                            return nx != 0 ? fma(A::WN(tabx, ix), gr, d) : d;
+                    };
+                    const bool forced = GUO || gto != T(0);
+                    if constexpr (QX >= 16) {
+                        if (forced) {
 #pragma unroll
-                    for (int ix = 0; ix < QX; ++ix) d[ix] = fma(ex[ix], rey, -f[k][ix]);
-                    if (GUO || gto != T(0)) {
+                            for (int ix = 0; ix < QX; ++ix)
+                                store(ix, force(ix, fma(ex[ix], rey, -f[k][ix])));
+                        } else {
 #pragma unroll
-                        for (int ix = 0; ix < QX; ++ix) {
-                            const int nx = AX::vel(ix);
-                            if constexpr (GUO)
-                                d[ix] = fma(A::W(tabx, ix), fma(T(nx), grA, T(AX::ck(ix)) * grB), d[ix]);
-                            else if (nx != 0)
-                                d[ix] = fma(A::WN(tabx, ix), gr, d[ix]);
+                            for (int ix = 0; ix < QX; ++ix) store(ix, fma(ex[ix], rey, -f[k][ix]));
                         }
-                    }
+                    } else {
+                        T d[QX];
 #pragma unroll
-                    for (int ix = 0; ix < QX; ++ix) op[ix * plane] = fma(om, d[ix], f[k][ix]);
+                        for (int ix = 0; ix < QX; ++ix) d[ix] = fma(ex[ix], rey, -f[k][ix]);
+                        if (forced) {
+#pragma unroll
+                            for (int ix = 0; ix < QX; ++ix) d[ix] = force(ix, d[ix]);
+                        }
+#pragma unroll
+                        for (int ix = 0; ix < QX; ++ix) store(ix, d[ix]);
+                    }
                 }
 #pragma unroll
                 for (int ix = (DEV ? QX - (QX & 1) : QX); ix < QX; ++ix) {
