@@ -5,7 +5,7 @@
 // copies: ping-pong). Every instance has its own geometry record (level,
 // nodes, pitch, offset into the pool). A uniform context (every instance
 // alike) is stepped by one launch of the tile kernel with the instance as the
-// grid's third dimension; a heterogeneous one by a persistent kernel over a
+// grid's third dimension; a heterogeneous one by one launch per level over a
 // work list of (instance, tile) items.
 #include <math.h>
 #include <stdarg.h>
@@ -238,8 +238,9 @@ static void fill_inst(const glbm_ctx *c, const glbm_config &cfg, const Geo &g, I
     for (int i = 0; i < ax_q(tabx); ++i) {
         double vp = 1.0;
         for (int p = 0; p < 4; ++p, vp *= ax_vel(tabx, i)) {
-            ip.kw_lo[p] += ip.ew_lo[i] * vp;
-            ip.kw_hi[p] += ip.ew_hi[i] * vp;
+            // (fused by name: the compiler's own choice moves with the code around it)
+            ip.kw_lo[p] = fma(ip.ew_lo[i], vp, ip.kw_lo[p]);
+            ip.kw_hi[p] = fma(ip.ew_hi[i], vp, ip.kw_hi[p]);
         }
     }
     ip.g_theta_om = ip.g_theta / ip.omega;
@@ -696,9 +697,9 @@ static int ctx_tile_shapes(const glbm_ctx *c, int N, TileShape *out)
 // most SMALL_WARPS warps (three per SM sub-partition), and more by the factor that
 // the tiles' 32-column rows waste on a lattice narrower than 16 columns. Measured
 // (GB300, D2Q81 unless noted, us per step, tiles -> small): 40 x 24 (270 warps)
-// 20.4 -> 8.6, 64 x 64 (1152) 20.3 -> 14.6, 128 x 64 (2304) 20.4 -> 24.3, 8 x 100
+// 20.4 -> 8.0, 64 x 64 (1152) 20.3 -> 14.6, 128 x 64 (2304) 20.4 -> 24.3, 8 x 100
 // 22.1 -> 8.2; D2Q289 4 x 60 44.4 -> 17.4; D1Q3 x D1Q28 5 instances of 1 x 200 106.6
-// -> 14.0. Choosing a tile shape, a wall-density mode or a dataflow mode afterwards
+// -> 12.7. Choosing a tile shape, a wall-density mode or a dataflow mode afterwards
 // takes the tiles (the results are the same).
 static const long long SMALL_WARPS = 3 * 608;
 static glbm_status choose_small(glbm_ctx *c)
