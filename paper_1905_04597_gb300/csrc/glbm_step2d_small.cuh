@@ -15,7 +15,7 @@
 // Every sum is taken in the order of the tile with G0 warp groups (the level's
 // default) and of k_wall_rho, so the results are those of the tiles bit for bit.
 // Measured on GB300, us per step in 64-step graphs, against the tiles: D2Q81 40 x 24
-// 20.4 -> 8.6, D1Q3 x D1Q28 5 x (1 x 200) 106.6 -> 14.0 (choose_small, glbm_api.cpp).
+// 20.4 -> 8.0, D1Q3 x D1Q28 5 x (1 x 200) 106.6 -> 12.7 (choose_small, glbm_api.cpp).
 #pragma once
 #include "glbm_step2d_launch.cuh"
 
