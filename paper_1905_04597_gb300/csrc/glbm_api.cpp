@@ -146,6 +146,7 @@ struct glbm_ctx {
     int4 *d_items = nullptr;       // heterogeneous work list, sorted by level
     int n_items = 0;
     int group[GLBM_MAXN + 2] = {0};  // first item of each level
+    long long pops[GLBM_MAXN + 1] = {0};  // populations of each level (batches)
     int tile[GLBM_MAXN + 1] = {0};   // tile shape index per level (glbm_tiles.h)
     bool small = false;              // steps with glbm_step2d_small.cuh
     AxisTableHi *d_tabs = nullptr;   // the axes' tables (y, x) of a small context
@@ -798,6 +799,7 @@ extern "C" glbm_status glbm_batch_create(const glbm_config *cfgs, int n, void *s
     if (!c) return fail(GLBM_E_NOMEM, "host allocation failed");
     c->hetero = true;
     glbm_status st = finish_create(c, cfgs, n, stream);
+    for (const Geo &g : c->geo) c->pops[g.N] += g.Q * g.nodes();
     if (st == GLBM_OK) choose_batch_tiles(c);
     if (st == GLBM_OK) st = create_side_streams(c);
     if (st == GLBM_OK) st = build_items(c);
@@ -1057,7 +1059,7 @@ static BatchArgs batch_args(const glbm_ctx *c, const void *fin, void *fout)
     b.n_items = c->n_items;
     for (int N = 0; N <= GLBM_MAXN + 1; ++N) b.group[N] = c->group[N];
     for (int N = 0; N <= GLBM_MAXN; ++N) b.shape[N] = c->tile[N];
-    for (const Geo &g : c->geo) b.pops[g.N] += g.Q * g.nodes();
+    for (int N = 0; N <= GLBM_MAXN; ++N) b.pops[N] = c->pops[N];
     b.status = c->d_status;
     b.step_ctr = c->d_status + ST_CLOCK;
     b.done_ctr = c->d_status + ST_DONE;
